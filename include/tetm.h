@@ -254,9 +254,12 @@ int tetm_set_kernel(tetm_solver* s, int32_t kernel);
  * way); each gives TETM_E_UNSUPPORTED for the other kind of solve and in
  * float64; the float32 defaults, chunk 32);
  * tile_x = 28 the warp-tiled kernel (one warp per item, tile_y in {4, 8,
- * 12, 16, 20, 28};
- * the float64 default, 28 x 20 x 32); tile_x = 32 (tile_y in {4, 8, 16}) or
- * 64 (tile_y in {4, 8}) the block-tiled kernel (one material only). Any value
+ * 12, 16, 20, 28}); tile_x = 32 (tile_y in {4, 8, 16}) or
+ * 64 (tile_y in {4, 8}) the block-tiled kernel (one material only). A float64
+ * solve whose shape was never set steps in two launches, one per half of the
+ * step, over bands of rows of every plane (not a z-slab, which runs the
+ * warp-tiled kernel; the shape reported, 28 x 20 x 32, is then the one the
+ * balances walk); the fields are the same bits on all of them. Any value
  * 0 keeps the current one. TETM_E_ARG for other values. */
 int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chunk_z);
 

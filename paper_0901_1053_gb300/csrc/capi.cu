@@ -367,6 +367,30 @@ int tetm::rebuild_work(tetm_solver* s) {
 
 namespace {
 
+// Work items of the float64 band kernels: the column hulls of the active
+// entries per (plane, band) from the device, the list from them.
+int build_band(tetm_solver* s) {
+  const int rows = band_rows(s->active_cells);
+  const size_t n = (size_t)((s->L.ny + rows - 1) / rows) * (size_t)s->L.nz;
+  int2* d = nullptr;
+  CK(dev_alloc((void**)&d, sizeof(int2) * n, s->stream));
+  std::vector<int2> h(n);
+  cudaError_t e = launch_band_hulls(s->mask, s->L, rows, d, s->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(int2) * n, cudaMemcpyDeviceToHost, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  dev_free(d, s->stream);
+  if (e != cudaSuccess) return cuda_fail(e);
+  std::vector<int4> items;
+  band_list(s->L, rows, h, &items, &s->band_smem);
+  s->n_band = (int)items.size();
+  if (items.empty()) return TETM_OK;
+  const int rc = dalloc(s, (void**)&s->band, sizeof(int4) * items.size());
+  if (rc != TETM_OK) return rc;
+  CK(cudaMemcpyAsync(s->band, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s->stream));
+  CK(cudaStreamSynchronize(s->stream));
+  return TETM_OK;
+}
+
 }  // namespace
 
 template <typename T>
@@ -518,7 +542,11 @@ int do_steps(tetm_solver* s, int n) {
     } else if (s->kernel == TETM_KERNEL_FUSED) {
       StepArgs<T> a = step_args<T>(s, true);
       if (s->n_work > 0) {
-        if (warp_shape_ok(s->tile_x, s->tile_y)) {
+        bool band = false;
+        if constexpr (sizeof(T) == 8) band = s->band && !s->own_shape;
+        if (band) {
+          if constexpr (sizeof(T) == 8) CK(launch_band_step(a, s->band, s->n_band, s->band_smem, s->stream));
+        } else if (warp_shape_ok(s->tile_x, s->tile_y)) {
           CK(launch_fused_warp_step<T>(a, s->tile_x, s->tile_y, s->stream));
         } else if (slab_shape_ok(s->tile_x, s->tile_y, !s->uniform)) {
           if constexpr (sizeof(T) == 4) {
@@ -610,6 +638,7 @@ void free_all(tetm_solver* s) {
   }
   dev_free(s->mask, st);
   dev_free(s->work, st);
+  dev_free(s->band, st);
   dev_free(s->J, st);
   dev_free(s->W, st);
   dev_free(s->qline, st);
@@ -814,6 +843,8 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
     s->active_cells = (long long)h;
   }
   if (rc == TETM_OK) rc = rebuild_work(s);
+  // (a z-slab keeps the fused sweep, which recomputes its ghost plane's TM half)
+  if (rc == TETM_OK && s->esz == 8 && !s->is_slab()) rc = build_band(s);
   if (rc != TETM_OK) {
     free_all(s);
     delete s;
@@ -911,6 +942,7 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   // the slab kernel is float32 only
   if ((slab_u || slab_m) && s->esz != 4) return TETM_E_UNSUPPORTED;
   if (s->kernel == TETM_KERNEL_TWOSTEP && !fused2_shape_ok(tx, ty)) return TETM_E_UNSUPPORTED;
+  if (tile_x || tile_y || chunk_z) s->own_shape = true;
   if (tx == s->tile_x && ty == s->tile_y && cz == s->chunk_z && s->work) return TETM_OK;
   s->tile_x = tx;
   s->tile_y = ty;

@@ -153,6 +153,14 @@ cudaError_t launch_fused_slab_batch(BatchMember<float>* members, int n_members, 
 // (a.co.ua[0] set: the per-entry coefficient arrays of material runs)
 cudaError_t launch_fused_slab_step(const StepArgs<float>& a, int* sched, cudaStream_t st);
 
+// ---- float64 step in two launches over bands of planes (kernels_band.cu) ---
+// the work items: int4 {plane, first row, first column, columns | rows << 16},
+// made from the column hull of the active entries of every (plane, band)
+int band_rows(long long active_cells);
+cudaError_t launch_band_hulls(const uint8_t* mask, const Layout& L, int rows, int2* out, cudaStream_t st);
+void band_list(const Layout& L, int rows, const std::vector<int2>& hulls, std::vector<int4>* items, int* smem);
+cudaError_t launch_band_step(const StepArgs<double>& a, const int4* items, int n, int smem, cudaStream_t st);
+
 // ---- Yee's E/M leapfrog, Eq. (7) (kernels_yee.cu): the step arguments carry
 // dt M^-1 as the per-component constants --------------------------------------
 template <typename T>
@@ -254,6 +262,9 @@ struct tetm_solver {
   int tiles_x, tiles_y, n_chunks;
   int* work;
   int n_work;
+  bool own_shape;              // the caller chose the work shape (tetm_set_tiling)
+  int4* band;                  // float64: work items of the band kernels (the default work shape)
+  int n_band, band_smem;
   std::vector<int> work_host;  // host copy of the work list
   bool in_batch;               // stepped by a tetm_batch
   bool work_dirty;
@@ -288,6 +299,29 @@ struct tetm_solver {
 };
 
 namespace tetm {
+// A launch that may begin before the kernel ahead of it in the stream has
+// ended: the kernel calls pdl_wait() before it reads or writes anything a
+// kernel ahead may write or read (what a solve never changes, its work list
+// and activity bytes, may be read before). pdl_trigger() in a kernel lets the
+// next such launch begin; it is called once every block runs, so the next
+// launch's blocks never take the place of blocks still to start.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // step arguments of a solve for the fused (ping-pong) or reference kernel
 template <typename T>
 StepArgs<T> step_args(tetm_solver* s, bool fused);
