@@ -56,6 +56,9 @@ extern "C" {
 #define TETM_RZ_KERNEL_BULK2 3     /* the bulk-copy sweep advancing two time steps per pass
                                       (temporal blocking: y^n read and y^{n+2} written once;
                                       an odd remaining step runs one-step)                  */
+/* A float64 solve for which neither a kernel nor a chunk length was ever set
+ * steps in two launches, one per half of the step, over runs of planes (the
+ * scattered-field form: on the default kernel); same results bit for bit. */
 
 typedef struct tetm_rz_grid {
   int32_t nr, nz;      /* primary cells, each >= 2                                 */

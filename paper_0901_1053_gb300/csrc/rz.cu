@@ -140,6 +140,7 @@ struct RzArgs {
   // work items [sc_lo, sc_hi) meet a source window: the kernels instantiated
   // with SC take exactly those, the plain ones skip them
   int sc_lo, sc_hi;
+  bool tm_only;           // mode 0: e_phi, h_r, h_z are zero (band kernels)
 };
 
 template <typename T>
@@ -918,6 +919,255 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) rz_step_bulk2_ker
   }
 }
 
+// --- float64 step in two launches over bands of planes -------------------------
+// The TM half (h_phi, h_r, e_z) of every plane, then the TE half (e_phi, e_r,
+// h_z). What bounds float64 is the float64 pipe (an instruction of a warp
+// takes the SM's pipe for 9.66 ns however many lanes are active; 31 of them
+// per 32 entries and step), so, as in the Cartesian band kernels: no march
+// along z (nothing computed twice, every run of planes independent), work
+// items cut to the columns between the first and last that carry a field, and
+// inside an item the entries of a stage dealt to the threads consecutively,
+// with the halo that stage needs (one column; planes need none). A work item is
+// a run of planes of one mode and its column range; intermediates stay in
+// shared memory. Mode 0 has no coupling between (e_r, e_z, h_phi), which the
+// bunch drives, and (e_phi, h_r, h_z): while nothing has set the latter they
+// are zero and neither read nor computed (RzArgs::tm_only). Per entry the
+// operations and their order are those of rz_plane, so the results are the
+// same bits. 256 x 2048, modes 0 and 1: 104.6 (asynchronous-copy sweep, 472
+// warps of 33 planes) -> 43.0 us a step; the float64 pipe alone takes 27.
+constexpr int kBandThreads = 256;
+constexpr int kBandMaxCols = 256;  // columns of an item at most
+
+// entry t of planes x width entries: t = thread, thread + kBandThreads, ...
+struct RzWalk {
+  int p, c;
+  const int w, planes;
+  __device__ __forceinline__ RzWalk(int planes_, int w_)
+      : p((int)threadIdx.x / w_), c((int)threadIdx.x % w_), w(w_), planes(planes_) {}
+  __device__ __forceinline__ bool ok() const { return p < planes; }
+  __device__ __forceinline__ void next() {
+    c += kBandThreads;
+    while (c >= w) {
+      c -= w;
+      ++p;
+    }
+  }
+};
+
+// values of shared memory of an item: two arrays of planes (w + 2), three of planes (w + 1)
+constexpr int rz_band_values(int planes, int w) { return planes * (5 * w + 7); }
+
+template <typename T>
+struct RzBand {
+  int mode, k0, planes, i0, w;  // owned: columns i0 .. i0 + w - 1 of planes k0 .. k0 + planes - 1
+  bool tm_only;
+  T mm;
+  const T* co;                  // coefficient row kCoER of (k0, i0)
+  const uint8_t* mask;          // mask entry of (i0, k0)
+  long long f;                  // field element of (mode, 0, i0, k0)
+};
+template <typename T>
+__device__ __forceinline__ RzBand<T> rz_band(const RzArgs<T>& a, const int4* items) {
+  const int4 v = items[blockIdx.x];
+  RzBand<T> b;
+  b.mode = blockIdx.y;
+  b.k0 = v.x;
+  b.planes = v.y;
+  b.i0 = v.z;
+  b.w = v.w;
+  b.mm = T(a.m_lo + b.mode);
+  b.tm_only = a.tm_only && a.m_lo + b.mode == 0;
+  b.co = a.coef + (long long)b.mode * a.co_mode + (long long)(v.x + 1) * a.co_plane + a.L.col(v.z);
+  b.mask = a.mask + a.L.midx(v.z, v.x);
+  b.f = a.L.fidx(b.mode, 0, v.z, v.x);
+  return b;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBandThreads, 4) rz_band_tm(const RzArgs<T> a, const int4* __restrict__ items) {
+  extern __shared__ __align__(16) unsigned char rz_band_sm[];
+  const RzBand<T> b = rz_band(a, items);
+  const long long PR = a.L.pr, RS = 6 * PR;
+  const int P = b.planes, W = b.w, w2 = W + 2, w1 = W + 1;
+  T* const hpa = reinterpret_cast<T*>(rz_band_sm);  // columns -1 .. W
+  T* const der = hpa + P * w2;
+  T* const hra = der + P * w2;                      // columns 0 .. W
+  T* const dep = hra + P * w1;
+  T* const ezn = dep + P * w1;
+  const T* __restrict__ in = a.in + b.f;
+  T* __restrict__ out = a.out + b.f;
+  tetm::pdl_trigger();
+  tetm::pdl_wait();
+  for (RzWalk t(P, w2); t.ok(); t.next()) {
+    const int c = t.c - 1;
+    const T* f = in + t.p * RS + 6 * c;
+    const unsigned m = b.mask[t.p * PR + c];
+    const T r0 = f[kER], r1 = f[RS + kER], z0 = f[kEZ], z1 = f[6 + kEZ], h0 = f[kHP];
+    T h = T(0), d = T(0);
+    if (m & 16) {
+      d = r1 - r0;
+      h = h0 + b.co[t.p * a.co_plane + kCoHP * PR + c] * (d - (z1 - z0));
+    }
+    hpa[t.p * w2 + t.c] = h;
+    der[t.p * w2 + t.c] = d;
+  }
+  if (!b.tm_only)
+    for (RzWalk t(P, w1); t.ok(); t.next()) {
+      const T* f = in + t.p * RS + 6 * t.c;
+      const unsigned m = b.mask[t.p * PR + t.c];
+      const T p0 = f[kEP], p1 = f[RS + kEP], z0 = f[kEZ], h0 = f[kHR];
+      T h = T(0), d = T(0);
+      if (m & 8) {
+        d = p1 - p0;
+        h = h0 + b.co[t.p * a.co_plane + kCoHR * PR + t.c] * (-d + b.mm * z0);
+      }
+      hra[t.p * w1 + t.c] = h;
+      dep[t.p * w1 + t.c] = d;
+    }
+  __syncthreads();
+  for (RzWalk t(P, w1); t.ok(); t.next()) {
+    const unsigned m = b.mask[t.p * PR + t.c];
+    const int i = b.i0 + t.c, k = b.k0 + t.p;
+    T e = T(0);
+    if (m & 4) {
+      const T* h = hpa + t.p * w2 + t.c + 1;
+      T cur = h[-1] - h[0];
+      if (!b.tm_only) cur = cur - b.mm * hra[t.p * w1 + t.c];
+      const bool line = a.b_on && i == a.i0;
+      if (line) {  // the bunch current on its ring
+        const long long dd = (long long)k - (a.n + a.kshift) + a.c0;
+        if (dd >= -a.c0 && dd < a.c0) cur -= a.J[(long long)b.mode * 2 * a.c0 + dd + a.c0];
+      }
+      const long long q = t.p * a.co_plane + t.c;
+      e = in[t.p * RS + 6 * t.c + kEZ] + b.co[q + ((m & 8) ? kCoFEZ : kCoEZ) * PR] * cur;
+      if (t.c < W) {
+        out[t.p * RS + 6 * t.c + kEZ] = e;
+        if (line) {
+          const long long w = (a.n + a.kshift) - k - a.c0 - a.m_min;
+          if (w >= 0 && w < a.nw)
+            a.W[((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w] -= (double)e * a.inv_q;
+        }
+      }
+    }
+    ezn[t.p * w1 + t.c] = e;
+  }
+  __syncthreads();
+  for (RzWalk t(P, W); t.ok(); t.next()) {
+    const unsigned m = b.mask[t.p * PR + t.c];
+    const long long q = t.p * a.co_plane + t.c;
+    const T* e = ezn + t.p * w1 + t.c;
+    T hp = T(0);
+    if (m & 16) {
+      hp = hpa[t.p * w2 + t.c + 1] + b.co[q + kCoHP * PR] * (der[t.p * w2 + t.c + 1] - (e[1] - e[0]));
+      out[t.p * RS + 6 * t.c + kHP] = hp;
+    }
+    if (!b.tm_only && (m & 8))
+      out[t.p * RS + 6 * t.c + kHR] =
+          hra[t.p * w1 + t.c] + b.co[q + kCoHR * PR] * (-dep[t.p * w1 + t.c] + b.mm * e[0]);
+    if (a.b_on && b.i0 + t.c == a.obs) {  // the transverse sample: old e_r, new h_phi
+      const long long w = (a.n + a.kshift) - (b.k0 + t.p) - a.c0 - a.m_min;
+      if (w >= 0 && w < a.nw)
+        a.WT[((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w] +=
+            a.tw_er * (double)in[t.p * RS + 6 * t.c + kER] + a.tw_hp * (double)hp;
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBandThreads, 4) rz_band_te(const RzArgs<T> a, const int4* __restrict__ items) {
+  extern __shared__ __align__(16) unsigned char rz_band_sm[];
+  const RzBand<T> b = rz_band(a, items);
+  const long long PR = a.L.pr, RS = 6 * PR;
+  const int P = b.planes, W = b.w, w2 = W + 2, w1 = W + 1;
+  const T* __restrict__ in = a.in + b.f;
+  T* __restrict__ out = a.out + b.f;  // h_phi, h_r as rz_band_tm left them
+  tetm::pdl_trigger();
+  tetm::pdl_wait();
+  if (b.tm_only) {
+    for (RzWalk t(P, W); t.ok(); t.next())
+      if (b.mask[t.p * PR + t.c] & 1) {
+        T* o = out + t.p * RS + 6 * t.c;
+        const T d = o[kHP - RS] - o[kHP], co = b.co[t.p * a.co_plane + kCoER * PR + t.c];
+        const T e = in[t.p * RS + 6 * t.c + kER] + co * -d;
+        o[kER] = e + co * -d;
+      }
+    return;
+  }
+  T* const epa = reinterpret_cast<T*>(rz_band_sm);  // columns -1 .. W
+  T* const dhr = epa + P * w2;
+  T* const era = dhr + P * w2;                      // columns -1 .. W-1
+  T* const dhp = era + P * w1;
+  T* const hzn = dhp + P * w1;
+  for (RzWalk t(P, w2); t.ok(); t.next()) {
+    const int c = t.c - 1;
+    const T* f = in + t.p * RS + 6 * c;
+    const T* o = out + t.p * RS + 6 * c;
+    const unsigned m = b.mask[t.p * PR + c];
+    const T h0 = o[kHR], h1 = o[kHR - RS], z0 = f[kHZ], z1 = f[kHZ - 6], e0 = f[kEP];
+    T e = T(0), d = T(0);
+    if (m & 2) {
+      d = h1 - h0;
+      e = e0 + b.co[t.p * a.co_plane + kCoEP * PR + c] * (d - (z1 - z0));
+    }
+    epa[t.p * w2 + t.c] = e;
+    dhr[t.p * w2 + t.c] = d;
+  }
+  for (RzWalk t(P, w1); t.ok(); t.next()) {
+    const int c = t.c - 1;
+    const T* f = in + t.p * RS + 6 * c;
+    const T* o = out + t.p * RS + 6 * c;
+    const unsigned m = b.mask[t.p * PR + c];
+    const T h0 = o[kHP], h1 = o[kHP - RS], z0 = f[kHZ], e0 = f[kER];
+    T e = T(0), d = T(0);
+    if (m & 1) {
+      d = h1 - h0;
+      e = e0 + b.co[t.p * a.co_plane + kCoER * PR + c] * (-d + b.mm * z0);
+    }
+    era[t.p * w1 + t.c] = e;
+    dhp[t.p * w1 + t.c] = d;
+  }
+  __syncthreads();
+  for (RzWalk t(P, w1); t.ok(); t.next()) {
+    const int c = t.c - 1;
+    const unsigned m = b.mask[t.p * PR + c];
+    T h = T(0);
+    if (m & 32) {
+      const T* e = epa + t.p * w2 + t.c;
+      const long long q = t.p * a.co_plane + c;
+      h = in[t.p * RS + 6 * c + kHZ] +
+          b.co[q + ((m & 1) ? kCoFHZ : kCoHZ) * PR] * ((e[1] - e[0]) - b.mm * era[t.p * w1 + t.c]);
+      if (t.c > 0) out[t.p * RS + 6 * c + kHZ] = h;
+    }
+    hzn[t.p * w1 + t.c] = h;
+  }
+  __syncthreads();
+  for (RzWalk t(P, W); t.ok(); t.next()) {
+    const unsigned m = b.mask[t.p * PR + t.c];
+    const long long q = t.p * a.co_plane + t.c;
+    const T* h = hzn + t.p * w1 + t.c + 1;
+    T* o = out + t.p * RS + 6 * t.c;
+    if (m & 1) o[kER] = era[t.p * w1 + t.c + 1] + b.co[q + kCoER * PR] * (-dhp[t.p * w1 + t.c + 1] + b.mm * h[0]);
+    if (m & 2)
+      o[kEP] = epa[t.p * w2 + t.c + 1] + b.co[q + kCoEP * PR] * (dhr[t.p * w2 + t.c + 1] - (h[-1] - h[0]));
+  }
+}
+
+// First and last + 1 column with an active entry of plane k (one warp each)
+__global__ void rz_plane_hulls(const uint8_t* mask, RzLayout L, int2* out) {
+  const int lane = threadIdx.x & 31;
+  const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (k >= L.nz) return;
+  int lo = L.nr + 1, hi = 0;
+  for (int i = lane; i <= L.nr; i += 32)
+    if (mask[L.midx(i, (int)k)]) {
+      lo = min(lo, i);
+      hi = max(hi, i + 1);
+    }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) out[k] = make_int2(lo, max(lo, hi));
+}
+
 // Scattered-field form. The incident field is the discrete TEM field of the
 // ring bunch in the entry pipe (the static start's field), continued along
 // the grid and moving one plane per step: at step n it is the static-start
@@ -1451,6 +1701,10 @@ struct tetm_rz {
   long long me_mode = 0, me_plane = 0;  // the same for metric
   int* work = nullptr;
   int n_work = 0, tiles = 0, chunk_z = 32, n_chunks = 0;
+  bool own_shape = false;        // the caller chose a kernel or a chunk length
+  int4* band = nullptr;          // float64: work items of the band kernels
+  int n_band = 0, band_smem = 0;
+  bool te_zero = true;           // nothing has set e_phi, h_r, h_z of mode 0
   bool work_dirty = true;
   long long processed = 0;
   int* flags = nullptr;
@@ -1613,6 +1867,8 @@ int rz_launch_steps(tetm_rz* s, long long n) {
   } else {
     a.tw_er = a.tw_hp = 0.0;
   }
+  a.tm_only = s->te_zero;
+  const bool band = s->band && !s->own_shape && !s->scattered;  // (the source windows are the other kernels')
   const int items = s->n_work * s->n_modes;
   const int blocks = std::max(1, std::min(s->resident, (items + 3) / 4));
   // launches one step kernel over the plain items (SC = false) or over the
@@ -1667,7 +1923,13 @@ int rz_launch_steps(tetm_rz* s, long long n) {
         a.sc_hi = s->chunk_first[(size_t)c_hi] * s->n_modes;
       }
     }
-    if (items > 0) {
+    if (band) {
+      cudaError_t e = tetm::launch_pdl(rz_band_tm<T>, dim3(s->n_band, s->n_modes), kBandThreads, s->band_smem, s->st,
+                                       a, s->band);
+      if (e == cudaSuccess)
+        e = tetm::launch_pdl(rz_band_te<T>, dim3(s->n_band, s->n_modes), kBandThreads, s->band_smem, s->st, a, s->band);
+      if (e != cudaSuccess) return rz_fail(e);
+    } else if (items > 0) {
       const bool win = a.sc_hi > a.sc_lo;
       if (win && !s->side) {  // the side stream and its two events, once
         if (cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1793,6 +2055,59 @@ int rz_rebuild_work(tetm_rz* s) {
   s->processed = processed * s->n_modes;
   s->work_dirty = false;
   return TETM_OK;
+}
+
+// Work items of the float64 band kernels {first plane, planes, first column,
+// columns}: runs of planes with about as many entries as the size of the
+// solve asks for, their columns between the first and last active one.
+int rz_build_band(tetm_rz* s) {
+  const RzLayout& L = s->L;
+  int2* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, sizeof(int2) * (size_t)L.nz);
+  if (e != cudaSuccess) return rz_fail(e);
+  std::vector<int2> h((size_t)L.nz);
+  rz_plane_hulls<<<(L.nz + 7) / 8, 256, 0, s->st>>>(s->mask, L, d);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(int2) * h.size(), cudaMemcpyDeviceToHost, s->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+  cudaFree(d);
+  if (e != cudaSuccess) return rz_fail(e);
+  long long total = 0;
+  for (const int2& v : h) total += v.y - v.x;
+  // about six items an SM, of 128 to 512 entries: 256 x 2048 with modes 0, 1
+  // takes 46.9 us a step with runs of 128 entries, 43.4 with 256, 42.8 with
+  // 512 and 57.3 with 1024 (0.64 M active entries)
+  const long long target = std::min(512LL, std::max(128LL, total * s->n_modes / (152 * 6)));
+  std::vector<int4> items;
+  int top = 0;
+  for (int k = 0; k < L.nz;) {
+    int lo = h[(size_t)k].x, hi = h[(size_t)k].y, n = 1;
+    if (hi > lo) {  // further planes while the run stays within the target and 64 planes
+      while (k + n < L.nz && n < 64) {
+        const int2 v = h[(size_t)(k + n)];
+        const int l2 = v.y > v.x ? std::min(lo, v.x) : lo, h2 = v.y > v.x ? std::max(hi, v.y) : hi;
+        // (a wider union than either plane's own range would deal out entries that carry nothing)
+        if ((long long)(n + 1) * std::min(h2 - l2, kBandMaxCols) > target || h2 - l2 > v.y - v.x + 8 ||
+            h2 - l2 > hi - lo + 8)
+          break;
+        lo = l2;
+        hi = h2;
+        ++n;
+      }
+      const int segs = (hi - lo + kBandMaxCols - 1) / kBandMaxCols, w = (hi - lo + segs - 1) / segs;
+      for (int i = lo; i < hi; i += w) {
+        items.push_back(make_int4(k, n, i, std::min(w, hi - i)));
+        top = std::max(top, rz_band_values(n, std::min(w, hi - i)));
+      }
+    }
+    k += n;
+  }
+  s->n_band = (int)items.size();
+  s->band_smem = top * s->esz;
+  if (items.empty()) return TETM_OK;
+  e = cudaMalloc(&s->band, sizeof(int4) * items.size());
+  if (e == cudaSuccess) e = cudaMemcpy(s->band, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? TETM_OK : rz_fail(e);
 }
 
 // Per-radian metric of one mode at radial index i (unscaled M^-1; zero where
@@ -2020,6 +2335,7 @@ int tetm_rz_create(const tetm_rz_grid* g, const double* eps_r, const double* mu_
   }
   if (rc == TETM_OK) rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
   if (rc == TETM_OK) rc = rz_rebuild_work(s);
+  if (rc == TETM_OK && s->esz == 8) rc = rz_build_band(s);
   if (rc != TETM_OK) {
     tetm_rz_destroy(s);
     return rc;
@@ -2447,12 +2763,14 @@ int tetm_rz_set_fields(tetm_rz* s, int32_t mode, int32_t comp, const double* in)
   cudaFreeAsync(tmp, s->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   s->prev_valid = false;
+  if (s->g.m_lo + mode == 0 && (comp == kEP || comp == kHR || comp == kHZ)) s->te_zero = false;
   return e == cudaSuccess ? TETM_OK : rz_fail(e);
 }
 
 int tetm_rz_set_tiling(tetm_rz* s, int32_t chunk_z) {
   if (!s || chunk_z < 4 || chunk_z > (1 << 20)) return TETM_E_ARG;
   s->chunk_z = chunk_z;
+  s->own_shape = true;
   s->work_dirty = true;
   return rz_rebuild_work(s);
 }
@@ -2464,6 +2782,7 @@ int tetm_rz_set_kernel(tetm_rz* s, int32_t kernel) {
   if (s->mat && kernel != TETM_RZ_KERNEL_REGISTER) return TETM_E_UNSUPPORTED;  // per-plane coefficients
   const bool retile = (kernel == TETM_RZ_KERNEL_BULK2) != (s->kernel == TETM_RZ_KERNEL_BULK2);
   s->kernel = kernel;
+  s->own_shape = true;
   int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
   if (rc == TETM_OK && retile) rc = rz_rebuild_work(s);
   return rc;
@@ -2630,6 +2949,7 @@ int tetm_rz_load(tetm_rz* s, const void* buf, size_t size) {
   if (e != cudaSuccess) return rz_fail(e);
   s->step = h.step;
   s->prev_valid = false;
+  s->te_zero = false;
   s->sc_until = 0;  // the scattered form's sources are recomputed from the loaded step on
   return TETM_OK;
 }
@@ -2644,6 +2964,7 @@ int tetm_rz_destroy(tetm_rz* s) {
   cudaFree(s->coef);
   cudaFree(s->metric);
   cudaFree(s->work);
+  cudaFree(s->band);
   cudaFree(s->flags);
   cudaFree(s->J);
   cudaFree(s->W);
