@@ -56,9 +56,11 @@ extern "C" {
 #define TETM_RZ_KERNEL_BULK2 3     /* the bulk-copy sweep advancing two time steps per pass
                                       (temporal blocking: y^n read and y^{n+2} written once;
                                       an odd remaining step runs one-step)                  */
-/* A float64 solve for which neither a kernel nor a chunk length was ever set
- * steps in two launches, one per half of the step, over runs of planes (the
- * scattered-field form: on the default kernel); same results bit for bit. */
+/* Until a kernel or a chunk length is set, the library chooses: float64 solves
+ * step in two launches, one per half of the step, over runs of planes (the
+ * scattered-field form: on the default kernel); float32 solves of one material
+ * take pairs of steps on the two-step kernel and end a call on a single step;
+ * the chunk length follows from the size. Same results bit for bit. */
 
 typedef struct tetm_rz_grid {
   int32_t nr, nz;      /* primary cells, each >= 2                                 */

@@ -51,6 +51,7 @@ using tetm::kMu0;
 constexpr int kER = TETM_RZ_ER, kEP = TETM_RZ_EPHI, kEZ = TETM_RZ_EZ;
 constexpr int kHR = TETM_RZ_HR, kHP = TETM_RZ_HPHI, kHZ = TETM_RZ_HZ;
 constexpr double kPi = 3.14159265358979323846;
+constexpr int kDefaultChunk = 32;  // planes per work item where a kernel but no chunk length was chosen
 constexpr int kTile = 60;   // entries a warp owns (64-entry window minus 2 + 2 halo)
 constexpr int kTile2 = 56;  // the same for two steps per pass (4 + 4 halo)
 // scattered-field form: steps whose sources one launch computes (a power of 2)
@@ -140,6 +141,11 @@ struct RzArgs {
   // work items [sc_lo, sc_hi) meet a source window: the kernels instantiated
   // with SC take exactly those, the plain ones skip them
   int sc_lo, sc_hi;
+  // windows of 56 owned entries: bit (k + 1) of [tile][change_words] says that
+  // the activity bytes of plane k differ from plane k - 1 somewhere in the window
+  const unsigned* changes;
+  int change_words;
+  int* sched;             // two zero counters (rz_step_pair_kernel draws its items, and leaves them zero)
   bool tm_only;           // mode 0: e_phi, h_r, h_z are zero (band kernels)
 };
 
@@ -352,20 +358,20 @@ __device__ __forceinline__ LaneCo<T> lane_coefs(const RzArgs<T>& a, const Item<T
 // Bunch current at the lane's e_z entry of plane k (zero off the ring) and
 // the wake sample of the new e_z.
 template <typename T>
-__device__ __forceinline__ T current_at(const RzArgs<T>& a, const Item<T>& it, bool src, int k) {
+__device__ __forceinline__ T current_at(const RzArgs<T>& a, const Item<T>& it, bool src, int k, long long n) {
   if (!src || k < 0) return T(0);
-  const long long dd = (long long)k - (a.n + a.kshift) + a.c0;
+  const long long dd = (long long)k - (n + a.kshift) + a.c0;
   return (dd >= -a.c0 && dd < a.c0) ? a.J[(long long)it.mode * 2 * a.c0 + dd + a.c0] : T(0);
 }
 // Scattered-field form: add the step's source to the new values of plane k
 // (all lanes; the window of planes is warp-uniform).
 template <typename T>
-__device__ __forceinline__ void add_source(const RzArgs<T>& a, const Item<T>& it, int k, T* out) {
+__device__ __forceinline__ void add_source(const RzArgs<T>& a, const Item<T>& it, int k, T* out, long long n) {
   if (!a.S) return;
-  const long long w = (long long)k - (a.n + a.sc_off);
+  const long long w = (long long)k - (n + a.sc_off);
   if (w < 0 || w >= a.sc_len) return;
   const T* p =
-      a.S + ((((a.n & (kSourceSlots - 1)) * a.n_modes + it.mode) * a.sc_len + w) * a.L.pr + a.L.col(it.gi)) * 6;
+      a.S + ((((n & (kSourceSlots - 1)) * a.n_modes + it.mode) * a.sc_len + w) * a.L.pr + a.L.col(it.gi)) * 6;
 #pragma unroll
   for (int q = 0; q < 12; ++q) out[q] += p[q];
 }
@@ -375,21 +381,31 @@ __device__ __forceinline__ void add_source(const RzArgs<T>& a, const Item<T>& it
 // longitudinal wake takes e_z at the bunch ring; the radial transverse wake
 // (E_r - c mu0 H_phi) at r_{obs+1/2}, where per radian h_phi = -r H_phi.
 // W and WT are [parity of n][mode][nw]; a wake is the sum of its two halves.
+// A sample is one fire-and-forget addition: as a load, an addition and a store
+// the round trip to memory held up the warp at every plane of the wake window,
+// which made the items on the bunch ring the last to end (the pass with
+// 32-plane items took 67 us a step on 512 x 4096 with modes 0..4).
+__device__ __forceinline__ void add_sample(double* w, double v) { atomicAdd(w, v); }
+__device__ __forceinline__ double long_sample(double ez, double inv_q) { return -__dmul_rn(ez, inv_q); }
+__device__ __forceinline__ double trans_sample(double tw_er, double er, double tw_hp, double hp) {
+  return fma(tw_er, er, __dmul_rn(tw_hp, hp));
+}
 template <typename T>
 __device__ __forceinline__ void gather_wake(const RzArgs<T>& a, const Item<T>& it, int k,
-                                            const T* out, const T* er_old) {
+                                            const T* out, const T* er_old, long long n) {
   if (!it.own || !a.b_on) return;
-  const long long w = (a.n + a.kshift) - k - a.c0 - a.m_min;
+  const long long w = (n + a.kshift) - k - a.c0 - a.m_min;
   if (w < 0 || w >= a.nw) return;
   // even and odd steps accumulate into separate halves: a pass that takes
   // two steps writes step n and step n+1 samples from different work items
-  const long long par = (a.n & 1) * (long long)a.n_modes * a.nw;
+  const long long par = (n & 1) * (long long)a.n_modes * a.nw;
   const bool s[2] = {it.src0, it.src1};
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
-    if (s[e]) a.W[par + (long long)it.mode * a.nw + w] -= (double)out[6 * e + kEZ] * a.inv_q;
+    if (s[e]) add_sample(a.W + par + (long long)it.mode * a.nw + w, long_sample((double)out[6 * e + kEZ], a.inv_q));
     if (it.gi + e == a.obs)
-      a.WT[par + (long long)it.mode * a.nw + w] += a.tw_er * (double)er_old[e] + a.tw_hp * (double)out[6 * e + kHP];
+      add_sample(a.WT + par + (long long)it.mode * a.nw + w,
+                 trans_sample(a.tw_er, (double)er_old[e], a.tw_hp, (double)out[6 * e + kHP]));
   }
 }
 
@@ -432,12 +448,12 @@ __device__ __forceinline__ void rz_item_reg(const RzArgs<T>& a, int witem, int s
       if (k >= it.k1) break;
       T out[12], er_old[2];
       if constexpr (MAT) c = lane_coefs(a, it, k);
-      rz_plane(ring[u], ring[(u + 1) % R], c, mm, s, current_at(a, it, it.src0, k),
-               current_at(a, it, it.src1, k), out, er_old);
-      if (SC) add_source(a, it, k, out);
+      rz_plane(ring[u], ring[(u + 1) % R], c, mm, s, current_at(a, it, it.src0, k, a.n),
+               current_at(a, it, it.src1, k, a.n), out, er_old);
+      if (SC) add_source(a, it, k, out, a.n);
       if (it.own && k >= it.k0) {
         st_pair(op + (long long)(k + 1) * RS, out);
-        gather_wake(a, it, k, out, er_old);
+        gather_wake(a, it, k, out, er_old, a.n);
       }
       load(k + R, ring[u]);
     }
@@ -548,12 +564,12 @@ __device__ __forceinline__ void rz_item_async(const RzArgs<T>& a, int witem, int
     __syncwarp();
     fetch(k + 1, d1);
     T out[12], er_old[2];
-    rz_plane(d0, d1, c, mm, s, current_at(a, it, it.src0, k), current_at(a, it, it.src1, k), out,
+    rz_plane(d0, d1, c, mm, s, current_at(a, it, it.src0, k, a.n), current_at(a, it, it.src1, k, a.n), out,
              er_old);
-    if (SC) add_source(a, it, k, out);
+    if (SC) add_source(a, it, k, out, a.n);
     if (it.own && k >= it.k0) {
       st_pair(op + (long long)(k + 1) * RS, out);
-      gather_wake(a, it, k, out, er_old);
+      gather_wake(a, it, k, out, er_old, a.n);
     }
     d0 = d1;
   }
@@ -719,12 +735,12 @@ __device__ __forceinline__ bool rz_item_bulk(const RzArgs<T>& a, int witem, int 
     fetch(k + 1, d1);
     if (!__all_sync(0xffffffffu, ok)) break;
     T out[12], er_old[2];
-    rz_plane(d0, d1, c, mm, s, current_at(a, it, it.src0, k), current_at(a, it, it.src1, k), out,
+    rz_plane(d0, d1, c, mm, s, current_at(a, it, it.src0, k, a.n), current_at(a, it, it.src1, k, a.n), out,
              er_old);
-    if (SC) add_source(a, it, k, out);
+    if (SC) add_source(a, it, k, out, a.n);
     if (it.own && k >= it.k0) {
       st_pair(op + (long long)(k + 1) * RS, out);
-      gather_wake(a, it, k, out, er_old);
+      gather_wake(a, it, k, out, er_old, a.n);
     }
     d0 = d1;
   }
@@ -801,9 +817,6 @@ __device__ __forceinline__ bool rz_item_bulk2(const RzArgs<T>& a, int witem, int
   const int klast = it.k1;                  // last plane of step 1
   const int moff = wcol - mcol + 2 * lane;
   int issued = kfirst - 1, fetched = kfirst - 1;
-  // a second item view for step 2: same geometry, one step later
-  RzArgs<T> a2 = a;
-  a2.n = a.n + 1;
 
   auto issue = [&](int p) {
     if (p > klast + 1) return;
@@ -854,11 +867,11 @@ __device__ __forceinline__ bool rz_item_bulk2(const RzArgs<T>& a, int witem, int
     // step 1 at plane k
     Pair6<T> y1;
     T er_old[2];
-    rz_plane(d0, d1, c, mm, s1, current_at(a, it, it.src0, k), current_at(a, it, it.src1, k), y1.f,
+    rz_plane(d0, d1, c, mm, s1, current_at(a, it, it.src0, k, a.n), current_at(a, it, it.src1, k, a.n), y1.f,
              er_old);
-    if (SC) add_source(a, it, k, y1.f);
+    if (SC) add_source(a, it, k, y1.f, a.n);
     y1.m = d0.m;
-    if (k >= it.k0 && k < it.k1) gather_wake(a, it, k, y1.f, er_old);
+    if (k >= it.k0 && k < it.k1) gather_wake(a, it, k, y1.f, er_old, a.n);
     // step 2 at plane k - 1 (from step-1 planes k-1 and k)
     const int k2 = k - 1;
     if (k2 == it.k0 - 1) {
@@ -870,12 +883,12 @@ __device__ __forceinline__ bool rz_item_bulk2(const RzArgs<T>& a, int witem, int
     }
     if (k2 >= it.k0 - 1) {
       T y2[12], er_old2[2];
-      rz_plane(y1prev, y1, c, mm, s2, current_at(a2, it, it.src0, k2), current_at(a2, it, it.src1, k2),
+      rz_plane(y1prev, y1, c, mm, s2, current_at(a, it, it.src0, k2, a.n + 1), current_at(a, it, it.src1, k2, a.n + 1),
                y2, er_old2);
-      if (SC) add_source(a2, it, k2, y2);
+      if (SC) add_source(a, it, k2, y2, a.n + 1);
       if (it.own && k2 >= it.k0) {
         st_pair(op + (long long)(k2 + 1) * RS, y2);
-        gather_wake(a2, it, k2, y2, er_old2);
+        gather_wake(a, it, k2, y2, er_old2, a.n + 1);
       }
     }
     y1prev = y1;
@@ -916,6 +929,309 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) rz_step_bulk2_ker
       if (chunk * a.chunk_z + sub * kSubPlanes >= a.L.nz) continue;
     }
     if (!rz_item_bulk2<T, SC>(a, it_w, sub, wsm, phases)) return;
+  }
+}
+
+// --- two steps per pass, float32, packed arithmetic ----------------------------
+// rz_step_bulk2_kernel's pass (the same ring, windows, recomputed planes and
+// results, bit for bit) for the items outside the source windows, rewritten
+// for instruction issue, which bound it (67% of the issue slots, 236
+// instructions per window of 64 entries, plane and step, of which 62 are the
+// arithmetic):
+//  * a lane's two entries ride in register pairs and every update is one
+//    packed instruction (fma.rn.f32x2 and its kin round each half as the
+//    scalar instruction does);
+//  * the coefficients are masked by the activity bytes once and kept; a plane
+//    whose bytes differ from the plane's before anywhere in the window (the
+//    ends of a cavity; one bit per plane and window, RzArgs::changes) rebuilds
+//    them from the coefficient rows;
+//  * planes where this window holds neither bunch current nor a wake sample
+//    (a range of planes found once per item) skip both;
+//  * two planes per loop turn, so no state is moved between registers; the
+//    copies are whole lines per warp (cp.async), and those of a warp's next
+//    item, drawn from a counter, follow the current item's without a gap.
+// 512 x 4096, modes 0..4 (157 000 window planes a pass): 66 -> 31 M warp
+// instructions a pass, DRAM 1.03 of one read and one write of the fields;
+// 52 -> 41 us a step (8- and 16-plane items, the best of each), the scattered
+// form 56 -> 48. What is left is latency: twelve warps an SM, a chain of about
+// 18 dependent operations and four shuffles per plane and step. Compiled for
+// four blocks an SM it spills: 49 us.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float lo(f2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi(f2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// the pair one entry to the right / to the left (outside the window: another
+// lane's value, which only halo entries read)
+__device__ __forceinline__ f2 right2(f2 v) { return pk(hi(v), __shfl_down_sync(0xffffffffu, lo(v), 1)); }
+__device__ __forceinline__ f2 left2(f2 v) { return pk(__shfl_up_sync(0xffffffffu, hi(v), 1), lo(v)); }
+
+struct PairPlane {
+  f2 er, ep, ez, hr, hp, hz;
+};
+struct PairCo {
+  f2 er, ep, hr, hp, fez, fhz;
+};
+
+// Both stages of a plane (rz_plane's operations in its order): y its old
+// state, er1, ep1 the old e of the plane above, hr_p, hp_p the new h of the
+// plane below (replaced by this plane's); jj the bunch current (JJ).
+template <bool JJ>
+__device__ __forceinline__ void pair_plane(const PairPlane& y, f2 er1, f2 ep1, const PairCo& c, f2 mm, f2 nmm, f2 jj,
+                                           f2& hr_p, f2& hp_p, PairPlane& o) {
+  const f2 der = sub2(er1, y.er), ndep = sub2(y.ep, ep1);
+  const f2 hpa = fma2(c.hp, sub2(der, sub2(right2(y.ez), y.ez)), y.hp);
+  const f2 hra = fma2(c.hr, fma2(mm, y.ez, ndep), y.hr);
+  f2 cur = fma2(nmm, hra, sub2(left2(hpa), hpa));
+  if (JJ) cur = sub2(cur, jj);
+  o.ez = fma2(c.fez, cur, y.ez);
+  o.hp = fma2(c.hp, sub2(der, sub2(right2(o.ez), o.ez)), hpa);
+  o.hr = fma2(c.hr, fma2(mm, o.ez, ndep), hra);
+  const f2 dhr = sub2(hr_p, o.hr), ndhp = sub2(o.hp, hp_p);
+  const f2 epa = fma2(c.ep, sub2(dhr, sub2(left2(y.hz), y.hz)), y.ep);
+  const f2 era = fma2(c.er, fma2(mm, y.hz, ndhp), y.er);
+  o.hz = fma2(c.fhz, fma2(nmm, era, sub2(right2(epa), epa)), y.hz);
+  o.ep = fma2(c.ep, sub2(dhr, sub2(left2(o.hz), o.hz)), epa);
+  o.er = fma2(c.er, fma2(mm, o.hz, ndhp), era);
+  hr_p = o.hr;
+  hp_p = o.hp;
+}
+
+__device__ __forceinline__ PairCo pair_coefs(const RzArgs<float>& a, const Item<float>& it, unsigned m) {
+  const LaneCo<float> c = lane_coefs(a, it);
+  float v[6][2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const unsigned b = (m >> (8 * e)) & 0xFFu;
+    v[0][e] = (b & 1) ? c.er[e] : 0.f;
+    v[1][e] = (b & 2) ? c.ep[e] : 0.f;
+    v[2][e] = (b & 8) ? c.hr[e] : 0.f;
+    v[3][e] = (b & 16) ? c.hp[e] : 0.f;
+    v[4][e] = (b & 4) ? ((b & 8) ? c.fez[e] : c.ez[e]) : 0.f;
+    v[5][e] = (b & 32) ? ((b & 1) ? c.fhz[e] : c.hz[e]) : 0.f;
+  }
+  return {pk(v[0][0], v[0][1]), pk(v[1][0], v[1][1]), pk(v[2][0], v[2][1]),
+          pk(v[3][0], v[3][1]), pk(v[4][0], v[4][1]), pk(v[5][0], v[5][1])};
+}
+
+__device__ __forceinline__ void pair_gather(const RzArgs<float>& a, const Item<float>& it, int k, const PairPlane& o,
+                                            f2 er_old, long long n) {
+  const float out[12] = {lo(o.er), lo(o.ep), lo(o.ez), lo(o.hr), lo(o.hp), lo(o.hz),
+                         hi(o.er), hi(o.ep), hi(o.ez), hi(o.hr), hi(o.hp), hi(o.hz)};
+  const float er[2] = {lo(er_old), hi(er_old)};
+  gather_wake(a, it, k, out, er, n);
+}
+
+// the ring of a warp: kPairDepth planes of [lane][12] values, each lane's own
+constexpr int kPairDepth = 8;
+constexpr size_t kPairWarpBytes = (size_t)kPairDepth * 32 * 48;
+
+// Warps take the plain items (those outside [sc_lo, sc_hi), which
+// rz_step_bulk2_kernel<float, true> takes) in list order, the first by their
+// index and then whichever is next, drawn one item ahead; the copies of the
+// next item's first planes follow the current item's last without a gap.
+__global__ void __launch_bounds__(128, 3) rz_step_pair_kernel(const RzArgs<float> a) {
+  extern __shared__ __align__(128) unsigned char rz_pair_smem[];
+  constexpr int D = kPairDepth;
+  const int lane = threadIdx.x & 31;
+  const unsigned ring = smem_u32(rz_pair_smem + (size_t)(threadIdx.x >> 5) * kPairWarpBytes);
+  const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+  const int gap = a.sc_hi - a.sc_lo, n_items = a.n_work * a.n_modes - gap;
+  const long long RS = a.L.pr * 6, MS = a.L.pr;
+  const long long at = a.n + a.kshift;
+  const f2 z2 = 0ull;
+  int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);  // the item at hand (among the plain ones)
+  auto list_item = [&](int qi) { return item_of(a, qi < a.sc_lo ? qi : qi + gap); };
+
+  const float* src = nullptr;  // the lane's 16 bytes of each third of the next plane to copy (whole lines)
+  int left = 0;                // planes of that item still to copy
+  unsigned slot = 0;           // of the plane at hand
+  unsigned islot = 0;          // of the next plane to copy: at most 7 planes on
+  int ahead = 0;               // planes copied of the item after the one at hand
+  auto copies_of = [&](const Item<float>& it) {
+    const int kf = max(it.k0 - 2, -1);
+    src = a.in + it.fbase + (long long)(kf + 1) * RS - 8 * lane;
+    left = it.k1 + 2 - kf;  // step 1 on planes kf .. k1 reads up to k1 + 1
+  };
+  // one copy group: the next plane's copies, or nothing
+  auto issue_one = [&]() {
+    const unsigned d = ring + islot * (32 * 48) + 16 * lane;
+#pragma unroll
+    for (int v = 0; v < 3; ++v)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 512 * v), "l"(src + 128 * v) : "memory");
+    src += RS;
+    islot = (islot + 1) & (D - 1);
+    cp_async_commit();
+  };
+  auto issue = [&]() {
+    if (left > 0) {
+      --left;
+      ++ahead;
+      issue_one();
+    } else {
+      cp_async_commit();
+    }
+  };
+  auto fetch = [&](unsigned sl, PairPlane& d) {
+    const unsigned s = ring + sl * (32 * 48) + 48 * lane;
+    float v[12];
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                   : "=f"(v[4 * u]), "=f"(v[4 * u + 1]), "=f"(v[4 * u + 2]), "=f"(v[4 * u + 3]) : "r"(s + 16 * u));
+    d.er = pk(v[0], v[6]);
+    d.ep = pk(v[1], v[7]);
+    d.ez = pk(v[2], v[8]);
+    d.hr = pk(v[3], v[9]);
+    d.hp = pk(v[4], v[10]);
+    d.hz = pk(v[5], v[11]);
+  };
+
+  if (q < n_items) copies_of(list_item(q));
+  while (q < n_items) {
+    // up to seven groups from this item's first plane on, so that the group of
+    // a plane is at least the seventh youngest when it is waited for
+    for (int p = ahead; p < D - 1; ++p) issue();
+    int ticket = 0;
+    if (lane == 0) ticket = atomicAdd(a.sched, 1);
+    const Item<float> it = list_item(q);
+    const int kfirst = max(it.k0 - 2, -1), klast = it.k1;  // planes of step 1
+    float* op = a.out + it.fbase + (long long)(it.k0 + 1) * RS;  // of the next plane to store
+    const unsigned* chg = a.changes + (long long)it.tile * a.change_words;
+    auto mask_at = [&](int k) { return ld_mask2(a.mask + it.mbase + (long long)(k + 1) * MS); };
+    // planes with a current or a sample of either step in this window
+    const int wlo = it.tile * a.tile_w - a.halo;
+    const bool line = a.b_on && ((a.i0 >= wlo && a.i0 < wlo + 64) || (a.obs >= wlo && a.obs < wlo + 64));
+    const int busy_lo = line ? (int)max(at - a.c0 - (a.m_min + a.nw - 1), -2LL) : 1;
+    const int busy_hi = line ? (int)min(at + 4, (long long)a.L.nz + 1) : 0;
+    PairCo c = pair_coefs(a, it, mask_at(kfirst));  // of the plane below the current one
+    unsigned bits = chg[(kfirst + 1) >> 5] >> ((kfirst + 1) & 31) & ~1u;  // from plane k on (c holds the first's)
+    const float fm = float(a.m_lo + it.mode);
+    const f2 mm = pk(fm, fm), nmm = pk(-fm, -fm);
+    PairPlane dA, dB, yA, yB;
+    f2 h1r = z2, h1p = z2, h2r = z2, h2p = z2;  // new h of the plane below, steps 1 and 2
+    yA = yB = {z2, z2, z2, z2, z2, z2};
+    bool drawn = false;
+    cp_async_wait<D - 2>();
+    __syncwarp();
+    fetch(slot, dA);
+
+    auto draw = [&]() {
+      if (left == 0 && !drawn) {  // every plane of this item is copied or on its way: the next item's follow
+        drawn = true;
+        ahead = 0;
+        q = nwarps + __shfl_sync(0xffffffffu, ticket, 0);
+        if (q < n_items) copies_of(list_item(q));
+      }
+    };
+    auto advance = [&](PairPlane& dn) {
+      cp_async_wait<D - 2>();
+      __syncwarp();  // plane k+1 is in, and every lane has read plane k
+      slot = (slot + 1) & (D - 1);
+      fetch(slot, dn);
+    };
+    const unsigned own = it.own ? 1u : 0u;
+    auto store = [&](const PairPlane& y2) {
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.u32 p, %13, 0;\n"
+          " @p st.global.v4.f32 [%0], {%1,%2,%3,%4};\n @p st.global.v4.f32 [%0+16], {%5,%6,%7,%8};\n"
+          " @p st.global.v4.f32 [%0+32], {%9,%10,%11,%12};\n}" ::"l"(op),
+          "f"(lo(y2.er)), "f"(lo(y2.ep)), "f"(lo(y2.ez)), "f"(lo(y2.hr)), "f"(lo(y2.hp)), "f"(lo(y2.hz)),
+          "f"(hi(y2.er)), "f"(hi(y2.ep)), "f"(hi(y2.ez)), "f"(hi(y2.hr)), "f"(hi(y2.hp)), "f"(hi(y2.hz)), "r"(own)
+          : "memory");
+      op += RS;
+    };
+    // plane k of step 1 (old state d, the plane above into dn, new state into
+    // y) and plane k - 1 of step 2 (old state yp), with every case
+    auto turn = [&](int k, const PairPlane& d, PairPlane& dn, const PairPlane& yp, PairPlane& y) {
+      draw();
+      issue();
+      advance(dn);
+      const bool busy = k >= busy_lo && k <= busy_hi;
+      const int k2 = k - 1;
+      PairPlane y2;
+      PairCo cn = c;
+      if (bits & 1u) cn = pair_coefs(a, it, mask_at(k));
+      pair_plane<true>(d, dn.er, dn.ep, cn, mm, nmm,
+                       pk(current_at(a, it, it.src0, k, a.n), current_at(a, it, it.src1, k, a.n)), h1r, h1p, y);
+      if (k2 >= it.k0 - 1)
+        pair_plane<true>(yp, y.er, y.ep, c, mm, nmm,
+                         pk(current_at(a, it, it.src0, k2, a.n + 1), current_at(a, it, it.src1, k2, a.n + 1)), h2r, h2p,
+                         y2);
+      c = cn;
+      if (busy && k >= it.k0 && k < it.k1) pair_gather(a, it, k, y, d.er, a.n);
+      if (k2 >= it.k0) {
+        if (busy) pair_gather(a, it, k2, y2, yp.er, a.n + 1);
+        store(y2);
+      }
+      bits >>= 1;
+      if (((k + 2) & 31) == 0) bits = chg[(k + 2) >> 5];
+    };
+    // the same on a quiet plane: both steps on, same coefficients, no current,
+    // no sample, a plane to copy
+    auto quiet = [&](const PairPlane& d, PairPlane& dn, const PairPlane& yp, PairPlane& y) {
+      issue_one();
+      advance(dn);
+      PairPlane y2;
+      pair_plane<false>(d, dn.er, dn.ep, c, mm, nmm, z2, h1r, h1p, y);
+      pair_plane<false>(yp, y.er, y.ep, c, mm, nmm, z2, h2r, h2p, y2);
+      store(y2);
+    };
+    for (int k = kfirst; k <= klast;) {
+      if (k > it.k0) {
+        // quiet planes from k on: to the next changed plane (or the end of the
+        // word of bits), the busy range, the item's last plane
+        draw();
+        int n = min(min(bits ? __ffs(bits) - 1 : 32, 31 - ((k + 1) & 31)), min(klast - k + 1, left)) & ~1;
+        if (k <= busy_hi && k + n > busy_lo) n = k >= busy_lo ? 0 : (busy_lo - k) & ~1;
+        if (n > 0) {
+          k += n;
+          bits >>= n;
+          left -= n;
+          ahead += n;
+          do {
+            quiet(dA, dB, yA, yB);
+            quiet(dB, dA, yB, yA);
+            n -= 2;
+          } while (n > 0);
+          continue;
+        }
+      }
+      turn(k, dA, dB, yA, yB);
+      if (++k > klast) break;
+      turn(k, dB, dA, yB, yA);
+      ++k;
+    }
+    slot = (slot + 1) & (D - 1);  // past plane k1 + 1: the next item's first
+  }
+  cp_async_wait<0>();
+  if (lane == 0) {  // the last warp to end resets the counters for the next launch
+    __threadfence();
+    if (atomicAdd(a.sched + 1, 1) == nwarps - 1) {
+      atomicExch(a.sched, 0);
+      atomicExch(a.sched + 1, 0);
+    }
   }
 }
 
@@ -1045,7 +1361,7 @@ __global__ void __launch_bounds__(kBandThreads, 4) rz_band_tm(const RzArgs<T> a,
         if (line) {
           const long long w = (a.n + a.kshift) - k - a.c0 - a.m_min;
           if (w >= 0 && w < a.nw)
-            a.W[((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w] -= (double)e * a.inv_q;
+            add_sample(a.W + ((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w, long_sample((double)e, a.inv_q));
         }
       }
     }
@@ -1067,8 +1383,8 @@ __global__ void __launch_bounds__(kBandThreads, 4) rz_band_tm(const RzArgs<T> a,
     if (a.b_on && b.i0 + t.c == a.obs) {  // the transverse sample: old e_r, new h_phi
       const long long w = (a.n + a.kshift) - (b.k0 + t.p) - a.c0 - a.m_min;
       if (w >= 0 && w < a.nw)
-        a.WT[((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w] +=
-            a.tw_er * (double)in[t.p * RS + 6 * t.c + kER] + a.tw_hp * (double)hp;
+        add_sample(a.WT + ((a.n & 1) * (long long)a.n_modes + b.mode) * a.nw + w,
+                   trans_sample(a.tw_er, (double)in[t.p * RS + 6 * t.c + kER], a.tw_hp, (double)hp));
     }
   }
 }
@@ -1150,6 +1466,25 @@ __global__ void __launch_bounds__(kBandThreads, 4) rz_band_te(const RzArgs<T> a,
     if (m & 2)
       o[kEP] = epa[t.p * w2 + t.c + 1] + b.co[q + kCoEP * PR] * (dhr[t.p * w2 + t.c + 1] - (h[-1] - h[0]));
   }
+}
+
+// RzArgs::changes: one warp per (tile, word of 32 planes)
+__global__ void rz_mask_changes(const uint8_t* mask, RzLayout L, int tiles, int words, unsigned* out) {
+  const int lane = threadIdx.x & 31;
+  const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (q >= (long long)tiles * words) return;
+  const int tile = (int)(q / words), word = (int)(q % words);
+  const long long col = (long long)tile * kTile2 - 4 + L.orr + 2 * lane;  // even, as the pitch
+  unsigned bits = 0;
+  for (int b = 0; b < 32; ++b) {
+    const long long row = (long long)word * 32 + b;
+    bool d = row == 0;
+    if (row > 0 && row < L.rows)
+      d = *reinterpret_cast<const unsigned short*>(mask + row * L.pr + col) !=
+          *reinterpret_cast<const unsigned short*>(mask + (row - 1) * L.pr + col);
+    if (__any_sync(0xffffffffu, d)) bits |= 1u << b;
+  }
+  if (lane == 0) out[q] = bits;
 }
 
 // First and last + 1 column with an active entry of plane k (one warp each)
@@ -1258,8 +1593,6 @@ __global__ void __launch_bounds__(128) rz_source_kernel(RzArgs<T> a, RzIncident 
     }
     const LaneCo<T> c = lane_coefs(a, it);
     const T mm = T(a.m_lo + mode);
-    RzArgs<T> an = a;
-    an.n = n;
     RzIncident xi = x, xo = x;
     xi.n = n;
     xo.n = n + 1;
@@ -1289,7 +1622,7 @@ __global__ void __launch_bounds__(128) rz_source_kernel(RzArgs<T> a, RzIncident 
       p0.m = m_pipe;
       p1 = d1;
       p1.m = m_pipe;
-      const T j0 = current_at(an, it, it.src0, k), j1 = current_at(an, it, it.src1, k);
+      const T j0 = current_at(a, it, it.src0, k, n), j1 = current_at(a, it, it.src1, k, n);
       T out[12], ref[12], er_old[2];
       rz_plane(d0, d1, c, mm, sg, j0, j1, out, er_old);
       rz_plane(p0, p1, c, mm, sp, j0, j1, ref, er_old);
@@ -1700,7 +2033,9 @@ struct tetm_rz {
   long long co_mode = 0, co_plane = 0;  // strides of coef per mode and per plane row (0: one row for all)
   long long me_mode = 0, me_plane = 0;  // the same for metric
   int* work = nullptr;
-  int n_work = 0, tiles = 0, chunk_z = 32, n_chunks = 0;
+  int n_work = 0, tiles = 0, chunk_z = kDefaultChunk, n_chunks = 0;
+  unsigned* changes = nullptr;   // float32, windows of 56: planes whose activity changes (RzArgs::changes)
+  int change_words = 0;
   bool own_shape = false;        // the caller chose a kernel or a chunk length
   int4* band = nullptr;          // float64: work items of the band kernels
   int n_band = 0, band_smem = 0;
@@ -1725,7 +2060,7 @@ struct tetm_rz {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int resident = 0;
   int kernel = TETM_RZ_KERNEL_ASYNC;
-  int* err = nullptr;            // device error word of the bulk-copy kernel
+  int* err = nullptr;            // device error word of the bulk-copy kernels; [2], [3]: schedule counters
   int obs = 0;                   // transverse wake at r_{obs+1/2}
   long long kshift = 0;          // static start: head at plane step + kshift
   int tile_w = kTile;            // owned entries per window of the current work list
@@ -1766,6 +2101,14 @@ RzIncident rz_incident(const tetm_rz* s, long long n) {
 }
 
 constexpr int kSourcePlanes = 2;  // planes per source work item
+
+// The step kernel in use: until one is chosen, float32 solves of one material
+// take pairs of steps on the two-step sweep (512 x 4096, modes 0..4: 104 us a
+// step on the one-step asynchronous-copy sweep, 41 on pairs) and single steps
+// on the bulk-copy sweep over the same work list.
+int rz_kernel(const tetm_rz* s) {
+  return !s->own_shape && s->esz == 4 && !s->mat ? TETM_RZ_KERNEL_BULK2 : s->kernel;
+}
 
 // Sources of the scattered-field form for steps s->step .. s->step + n_steps - 1.
 template <typename T>
@@ -1867,7 +2210,11 @@ int rz_launch_steps(tetm_rz* s, long long n) {
   } else {
     a.tw_er = a.tw_hp = 0.0;
   }
+  const int kernel = rz_kernel(s);
   a.tm_only = s->te_zero;
+  a.changes = s->changes;
+  a.change_words = s->change_words;
+  a.sched = s->err + 2;
   const bool band = s->band && !s->own_shape && !s->scattered;  // (the source windows are the other kernels')
   const int items = s->n_work * s->n_modes;
   const int blocks = std::max(1, std::min(s->resident, (items + 3) / 4));
@@ -1876,11 +2223,14 @@ int rz_launch_steps(tetm_rz* s, long long n) {
   auto launch = [&](bool sc, int steps, int nblocks, cudaStream_t st) {
     if (steps == 2) {
       if (sc) rz_step_bulk2_kernel<T, true><<<nblocks, 128, 4 * rz_bulk_warp_bytes<T>(), st>>>(a);
-      else rz_step_bulk2_kernel<T, false><<<nblocks, 128, 4 * rz_bulk_warp_bytes<T>(), st>>>(a);
-    } else if (s->kernel == TETM_RZ_KERNEL_BULK || s->kernel == TETM_RZ_KERNEL_BULK2) {
+      else if constexpr (sizeof(T) == 4)
+        rz_step_pair_kernel<<<nblocks, 128, 4 * kPairWarpBytes, st>>>(a);
+      else
+        rz_step_bulk2_kernel<T, false><<<nblocks, 128, 4 * rz_bulk_warp_bytes<T>(), st>>>(a);
+    } else if (kernel == TETM_RZ_KERNEL_BULK || kernel == TETM_RZ_KERNEL_BULK2) {
       if (sc) rz_step_bulk_kernel<T, true><<<nblocks, 128, 4 * rz_bulk_warp_bytes<T>(), st>>>(a);
       else rz_step_bulk_kernel<T, false><<<nblocks, 128, 4 * rz_bulk_warp_bytes<T>(), st>>>(a);
-    } else if (s->kernel == TETM_RZ_KERNEL_ASYNC) {
+    } else if (kernel == TETM_RZ_KERNEL_ASYNC) {
       if (sc) rz_step_async_kernel<T, true><<<nblocks, 128, 4 * rz_async_warp_bytes<T>(), st>>>(a);
       else rz_step_async_kernel<T, false><<<nblocks, 128, 4 * rz_async_warp_bytes<T>(), st>>>(a);
     } else if (s->mat) {  // material arrays: the register kernel, coefficients per plane
@@ -1897,7 +2247,9 @@ int rz_launch_steps(tetm_rz* s, long long n) {
     a.n = s->step;
     // steps in this pass: two with the two-step kernel, except past or into
     // a step that carries balances (they need the state one step before it)
-    int p = (s->kernel == TETM_RZ_KERNEL_BULK2 && t + 1 < n) ? 2 : 1;
+    // (without a chosen kernel the last step is a single one, so that the call
+    // leaves the state before the last step in the other set)
+    int p = (kernel == TETM_RZ_KERNEL_BULK2 && t + (s->own_shape ? 1 : 2) < n) ? 2 : 1;
     if (p == 2 && s->bal_every > 0 &&
         ((s->step + 1) % s->bal_every == 0 || (s->step + 2) % s->bal_every == 0))
       p = 1;
@@ -1969,6 +2321,7 @@ int rz_launch_steps(tetm_rz* s, long long n) {
 // Blocks of 4 warps the step kernel keeps resident on the whole device.
 template <typename T>
 int rz_occupancy(tetm_rz* s) {
+  const int kernel = rz_kernel(s);
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1986,18 +2339,28 @@ int rz_occupancy(tetm_rz* s) {
   if (e == cudaSuccess && bsmem > 48 * 1024)
     e = cudaFuncSetAttribute(rz_step_bulk_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)bsmem);
-  if (e == cudaSuccess && bsmem > 48 * 1024)
-    e = cudaFuncSetAttribute(rz_step_bulk2_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bsmem);
+  if constexpr (sizeof(T) == 8) {  // (float32 pairs of steps: rz_step_pair_kernel)
+    if (e == cudaSuccess && bsmem > 48 * 1024)
+      e = cudaFuncSetAttribute(rz_step_bulk2_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)bsmem);
+  }
   if (e == cudaSuccess && bsmem > 48 * 1024)
     e = cudaFuncSetAttribute(rz_step_bulk2_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)bsmem);
+  if constexpr (sizeof(T) == 4) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(rz_step_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * kPairWarpBytes));
+  }
   if (e == cudaSuccess) {
-    if (s->kernel == TETM_RZ_KERNEL_BULK2)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_bulk2_kernel<T, false>, 128, bsmem);
-    else if (s->kernel == TETM_RZ_KERNEL_BULK)
+    if (kernel == TETM_RZ_KERNEL_BULK2) {
+      if constexpr (sizeof(T) == 4)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_pair_kernel, 128, 4 * kPairWarpBytes);
+      else
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_bulk2_kernel<T, false>, 128, bsmem);
+    }
+    else if (kernel == TETM_RZ_KERNEL_BULK)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_bulk_kernel<T, false>, 128, bsmem);
-    else if (s->kernel == TETM_RZ_KERNEL_ASYNC)
+    else if (kernel == TETM_RZ_KERNEL_ASYNC)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_async_kernel<T, false>, 128, smem);
     else
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rz_step_kernel<T, false>, 128, 0);
@@ -2009,7 +2372,7 @@ int rz_occupancy(tetm_rz* s) {
 
 int rz_rebuild_work(tetm_rz* s) {
   const RzLayout& L = s->L;
-  const int tw = s->kernel == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile;
+  const int tw = rz_kernel(s) == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile;
   s->tile_w = tw;
   s->tiles = (L.nr + 1 + tw - 1) / tw;
   s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
@@ -2050,11 +2413,36 @@ int rz_rebuild_work(tetm_rz* s) {
     e = cudaMemcpy(s->work, w.data(), sizeof(int) * w.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return rz_fail(e);
   }
+  if (s->esz == 4 && tw == kTile2 && !s->changes) {  // once: they depend on the geometry only
+    s->change_words = (int)((L.rows + 31) / 32);
+    const long long warps = (long long)s->tiles * s->change_words;
+    e = cudaMalloc(&s->changes, sizeof(unsigned) * (size_t)warps);
+    if (e != cudaSuccess) return rz_fail(e);
+    rz_mask_changes<<<(unsigned)((warps + 7) / 8), 256, 0, s->st>>>(s->mask, L, s->tiles, s->change_words, s->changes);
+    if ((e = cudaGetLastError()) != cudaSuccess) return rz_fail(e);
+  }
   s->n_work = (int)w.size();
   s->chunk_first[(size_t)s->n_chunks] = s->n_work;
   s->processed = processed * s->n_modes;
   s->work_dirty = false;
   return TETM_OK;
+}
+
+// Planes per work item until a length is chosen: about four items per resident
+// warp, within 2 .. 16 planes (long items amortise the planes each recomputes,
+// short ones spread a small solve and even out the end of the launch).
+// us a step on the pair kernel: 512 x 4096, modes 0..4 (130 000 window planes,
+// 1824 warps): 54 with 4 planes, 45 with 8, 41 with 16, 53 with 32, 67 with 48;
+// 93 x 771, mode 0 (1000 window planes): 7.6 with 4, 10.3 with 8, 28.7 with 32.
+int rz_default_chunk(tetm_rz* s) {
+  int rc = rz_rebuild_work(s);
+  if (rc != TETM_OK) return rc;
+  const long long planes = (long long)s->n_work * s->n_modes * s->chunk_z;
+  const long long least = s->esz == 8 ? 8 : s->mat ? 4 : 2;  // (the one-step sweeps start later)
+  const int cz = (int)std::min(16LL, std::max(least, planes / (4LL * 4 * std::max(1, s->resident)) / 2 * 2));
+  if (cz >= s->L.nz) return TETM_OK;
+  s->chunk_z = cz;
+  return rz_rebuild_work(s);
 }
 
 // Work items of the float64 band kernels {first plane, planes, first column,
@@ -2310,8 +2698,8 @@ int tetm_rz_create(const tetm_rz_grid* g, const double* eps_r, const double* mu_
     if ((e = cudaMalloc(&s->coef, cob)) != cudaSuccess) break;
     if ((e = cudaMalloc(&s->metric, meb)) != cudaSuccess) break;
     if ((e = cudaMalloc(&s->partial, sizeof(double) * (kEnergyBlocks + 1))) != cudaSuccess) break;
-    if ((e = cudaMalloc(&s->err, sizeof(int))) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(s->err, 0, sizeof(int), s->st)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&s->err, 4 * sizeof(int))) != cudaSuccess) break;
+    if ((e = cudaMemsetAsync(s->err, 0, 4 * sizeof(int), s->st)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(s->set[0], 0, fb, s->st)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(s->set[1], 0, fb, s->st)) != cudaSuccess) break;
     if (pec) {
@@ -2334,7 +2722,7 @@ int tetm_rz_create(const tetm_rz_grid* g, const double* eps_r, const double* mu_
     rc = s->esz == 8 ? rz_upload_coefs<double>(s) : rz_upload_coefs<float>(s);
   }
   if (rc == TETM_OK) rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
-  if (rc == TETM_OK) rc = rz_rebuild_work(s);
+  if (rc == TETM_OK) rc = rz_default_chunk(s);
   if (rc == TETM_OK && s->esz == 8) rc = rz_build_band(s);
   if (rc != TETM_OK) {
     tetm_rz_destroy(s);
@@ -2770,8 +3158,13 @@ int tetm_rz_set_fields(tetm_rz* s, int32_t mode, int32_t comp, const double* in)
 int tetm_rz_set_tiling(tetm_rz* s, int32_t chunk_z) {
   if (!s || chunk_z < 4 || chunk_z > (1 << 20)) return TETM_E_ARG;
   s->chunk_z = chunk_z;
+  const bool first = !s->own_shape;
   s->own_shape = true;
   s->work_dirty = true;
+  if (first) {  // the kernel may change with it
+    const int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
+    if (rc != TETM_OK) return rc;
+  }
   return rz_rebuild_work(s);
 }
 
@@ -2780,8 +3173,9 @@ int tetm_rz_set_kernel(tetm_rz* s, int32_t kernel) {
              kernel != TETM_RZ_KERNEL_BULK && kernel != TETM_RZ_KERNEL_BULK2))
     return TETM_E_ARG;
   if (s->mat && kernel != TETM_RZ_KERNEL_REGISTER) return TETM_E_UNSUPPORTED;  // per-plane coefficients
-  const bool retile = (kernel == TETM_RZ_KERNEL_BULK2) != (s->kernel == TETM_RZ_KERNEL_BULK2);
+  const bool retile = !s->own_shape || (kernel == TETM_RZ_KERNEL_BULK2) != (s->kernel == TETM_RZ_KERNEL_BULK2);
   s->kernel = kernel;
+  if (!s->own_shape) s->chunk_z = kDefaultChunk;
   s->own_shape = true;
   int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
   if (rc == TETM_OK && retile) rc = rz_rebuild_work(s);
@@ -2965,6 +3359,7 @@ int tetm_rz_destroy(tetm_rz* s) {
   cudaFree(s->metric);
   cudaFree(s->work);
   cudaFree(s->band);
+  cudaFree(s->changes);
   cudaFree(s->flags);
   cudaFree(s->J);
   cudaFree(s->W);
