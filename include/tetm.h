@@ -247,12 +247,14 @@ int tetm_set_kernel(tetm_solver* s, int32_t kernel);
 
 /* Fused-kernel work shape: transverse tile tile_x x tile_y and z-chunk
  * length chunk_z >= 4 of one work item. 56 x 28 selects the float32 slab
- * kernel for one material (one CTA of 512 threads per SM; e_z, h_z staged in
- * shared memory by per-thread asynchronous copies of the quads that carry
- * them), 56 x 12 the slab kernel for material arrays (two CTAs of 256
- * threads per SM; e_z, h_z and the six coefficient arrays staged the same
- * way); each gives TETM_E_UNSUPPORTED for the other kind of solve and in
- * float64; the float32 defaults, chunk 32);
+ * kernel for one material (e_z, h_z staged in shared memory by per-thread
+ * asynchronous copies of the quads that carry them), 56 x 12 the slab kernel
+ * for material arrays (e_z, h_z and the six coefficient arrays staged the same
+ * way); both run two CTAs of 256 threads per SM on work items of 56 x 12
+ * nodes; each gives TETM_E_UNSUPPORTED for the other kind of solve and in
+ * float64; the float32 defaults, with chunks of 4 to 64 planes chosen for the
+ * geometry so that the items fill the GPU in whole rounds until a chunk is
+ * set; in a batch for the member's share of it);
  * tile_x = 28 the warp-tiled kernel (one warp per item, tile_y in {4, 8,
  * 12, 16, 20, 28}); tile_x = 32 (tile_y in {4, 8, 16}) or
  * 64 (tile_y in {4, 8}) the block-tiled kernel (one material only). A float64

@@ -3,7 +3,7 @@
 // sizes fill the GPU; the member descriptors live on the device and are
 // advanced there (ping-pong swap, step count, retirement at the member's step
 // limit), which lets a run of steps be captured once as a CUDA graph and
-// replayed. Float32 batches on the slab kernel's tile (56 x 28) run the
+// replayed. Float32 batches on the slab kernel's shape (56 x 28) run the
 // batched slab kernel, the others the batched warp-tiled kernel.
 //
 // A batch is a table of slots. Members join and leave between step calls:
@@ -42,9 +42,10 @@ struct tetm_batch {
   int capacity;
   std::vector<tetm_solver*> slot;  // per slot: the member, or nullptr
   std::vector<long long> limit;    // per slot: the step index its member stops at
+  std::vector<std::vector<int>> items;  // per slot: the member's work items in this batch
   size_t esz;
   int tile_x, tile_y;
-  bool slab;                       // the batched slab kernel (float32, 56 x 28 tiles)
+  bool slab;                       // the batched slab kernel (float32, shape 56 x 28)
   void* d_members;                 // BatchMember<T>[capacity]
   int* d_wbuf;                     // kHead ints (entry count first), then int2 entries
   int wcap;                        // entries d_wbuf holds
@@ -130,7 +131,7 @@ int upload_work(tetm_batch* b) {
   for (int i = 0; i < b->capacity; ++i) {
     tetm_solver* s = b->slot[(size_t)i];
     if (!s || s->step >= b->limit[(size_t)i]) continue;
-    for (int item : s->work_host) {
+    for (int item : b->items[(size_t)i]) {
       h.push_back(i);
       h.push_back(item);
     }
@@ -253,6 +254,7 @@ int create_slots(int capacity, size_t esz, int tile_x, int tile_y, int graph_ste
   b->capacity = capacity;
   b->slot.assign((size_t)capacity, nullptr);
   b->limit.assign((size_t)capacity, 0);
+  b->items.resize((size_t)capacity);
   b->esz = esz;
   b->tile_x = tile_x;
   b->tile_y = tile_y;
@@ -313,6 +315,15 @@ int write_member(tetm_batch* b, int i, tetm_solver* s) {
   memset(&m, 0, sizeof(m));
   m.a = step_args<T>(s, true);
   m.a.work = nullptr;  // the batch's combined list is used instead
+  // in it the member's items have the length that suits a share of the GPU
+  // (choose_chunk), unless the caller set one; its own list stays as it is
+  std::vector<int>& items = b->items[(size_t)i];
+  items = s->work_host;
+  if (b->slab && !s->own_chunk && s->auto_chunk()) {
+    m.a.chunk_z = choose_chunk(s, b->capacity);
+    m.a.n_chunks = (s->L.nz + m.a.chunk_z - 1) / m.a.chunk_z;
+    work_list(s, m.a.chunk_z, &items);
+  }
   m.limit = b->limit[(size_t)i];
   m.active = s->step < b->limit[(size_t)i] ? 1 : 0;
   m.cur = s->cur;

@@ -186,27 +186,22 @@ __global__ void from_canonical(const double* src, Layout L, int k0, int nk, cons
   dst[id] = ((mask[id] >> comp) & 1) ? (T)src[q] : T(0);
 }
 
-// Per fused work item (tile, z-chunk): the number of its own cells that
-// carry a field (0: the item lies in PEC and is skipped).
-__global__ void item_counts(const uint8_t* mask, Layout L, int tx, int ty, int cz, int tiles_x,
-                            int tiles_y, int n_items, int* counts) {
-  __shared__ int total;
-  const int item = blockIdx.x;
-  if (item >= n_items) return;
-  if (threadIdx.x == 0) total = 0;
-  __syncthreads();
-  const int ntile = tiles_x * tiles_y;
-  const int tile = item % ntile, chunk = item / ntile;
-  const int i0 = (tile % tiles_x) * tx, j0 = (tile / tiles_x) * ty, k0 = chunk * cz;
-  int c = 0;
-  const int cells = tx * ty * cz;
-  for (int q = threadIdx.x; q < cells; q += blockDim.x) {
-    const int i = i0 + q % tx, j = j0 + (q / tx) % ty, k = k0 + q / (tx * ty);
-    if (i < L.nx && j < L.ny && k < L.nz && mask[L.idx(i, j, k)] != 0) ++c;
+// Per tile and plane (tile-major): 1 where one of the tile's own cells carries
+// a field in that plane; a warp per (tile, plane).
+__global__ void tile_activity(const uint8_t* mask, Layout L, int tx, int ty, int tiles_x, long long n,
+                              uint8_t* act) {
+  const int lane = threadIdx.x & 31;
+  const long long step = (long long)gridDim.x * blockDim.x / 32;
+  for (long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; q < n; q += step) {
+    const int tile = (int)(q / L.nz), k = (int)(q % L.nz);
+    const int i0 = (tile % tiles_x) * tx, j0 = (tile / tiles_x) * ty;
+    bool any = false;
+    for (int c = lane; c - lane < tx * ty && !any; c += 32) {
+      const int i = i0 + c % tx, j = j0 + c / tx;
+      any = __any_sync(0xffffffffu, c < tx * ty && i < L.nx && j < L.ny && mask[L.idx(i, j, k)] != 0);
+    }
+    if (lane == 0) act[q] = any ? 1 : 0;
   }
-  atomicAdd(&total, c);
-  __syncthreads();
-  if (threadIdx.x == 0) counts[item] = total;
 }
 
 // Entries of one component that hold a non-zero value where the activity bit
@@ -316,35 +311,92 @@ void tetm::dev_free(void* p, cudaStream_t st) {
   if (p) cudaFreeAsync(p, st);
 }
 
+// The items (tile, chunk of cz planes) that own a field-carrying cell, in grid
+// order: items that run at the same time are neighbours and share their halo
+// rows through L2 (ordering the list by work instead was measured 1.3x slower).
+void tetm::work_list(const tetm_solver* s, int cz, std::vector<int>* list) {
+  const int nz = s->L.nz, tiles = s->tiles_x * s->tiles_y;
+  list->clear();
+  for (int k0 = 0, c = 0; k0 < nz; k0 += cz, ++c)
+    for (int t = 0; t < tiles; ++t)
+      if (memchr(s->act.data() + (size_t)t * nz + k0, 1, (size_t)std::min(cz, nz - k0)))
+        list->push_back(c * tiles + t);
+}
+
+// Planes per work item of the slab kernel, where the caller set none. Every
+// item takes about cz + 2 planes' time (the plane below the chunk, and filling
+// the pipeline) and the GPU holds two per SM at once, so a step takes
+// ceil(items / slots) rounds of cz + 2 planes. Measured on eight one-material
+// geometries (48 x 48 x 192 to 256 x 256 x 1024, every cz of 4..24 and every
+// third to 62), the cz of the fewest such planes was the fastest in six, 1 and
+// 10% off in the others; in three material ones 0 to 6%. Against 32 planes
+// always: 32.8 -> 10.3 us per step on 48 x 48 x 192, 96.8 -> 63.5 on 128 x 128
+// x 600 (342 items at 32 planes are two rounds, 288 at 38 one).
+// Of `share` solves that step together each has its part of many rounds, so
+// the last one counts by half: items * share / slots + 1/2 on average, at least
+// one, and no more than kChunk planes, since the others may leave early (a batch
+// of 16: 406 ms at 20 to 32 planes, 441 at 8, 423 at 64).
+int tetm::choose_chunk(const tetm_solver* s, int share) {
+  const int nz = s->L.nz, tiles = s->tiles_x * s->tiles_y;
+  const int top = std::min(share == 1 ? kMaxChunk : kChunk, std::max(nz, kMinChunk));
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+    cudaGetLastError();
+    return kChunk;
+  }
+  const double slots = 2.0 * sms;
+  std::vector<long long> items((size_t)top + 1, 0);
+  std::vector<int> before((size_t)nz + 1);  // active planes of the tile below a plane
+  for (int t = 0; t < tiles; ++t) {
+    const uint8_t* a = s->act.data() + (size_t)t * nz;
+    before[0] = 0;
+    for (int k = 0; k < nz; ++k) before[(size_t)k + 1] = before[(size_t)k] + a[k];
+    if (!before[(size_t)nz]) continue;
+    for (int cz = kMinChunk; cz <= top; ++cz)
+      for (int k0 = 0; k0 < nz; k0 += cz)
+        items[(size_t)cz] += before[(size_t)std::min(k0 + cz, nz)] > before[(size_t)k0];
+  }
+  int best = kMinChunk;
+  double least = 0.0;
+  for (int cz = kMinChunk; cz <= top; ++cz) {
+    const double r = (double)items[(size_t)cz] * share / slots;
+    const double cost = (share == 1 ? ceil(r) : std::max(r + 0.5, 1.0)) * (cz + 2);
+    if (cz == kMinChunk || cost <= least) {  // of equals the longest: fewest planes read twice
+      best = cz;
+      least = cost;
+    }
+  }
+  return best;
+}
+
 int tetm::rebuild_work(tetm_solver* s) {
   const Layout& L = s->L;
   s->tiles_x = (L.nx + s->tile_x - 1) / s->tile_x;
-  s->tiles_y = (L.ny + s->tile_y - 1) / s->tile_y;
-  s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
-  const long long items = (long long)s->tiles_x * s->tiles_y * s->n_chunks;
-  if (items >= (1LL << 31)) return TETM_E_ARG;
+  const int rows = slab_rows(s->tile_x, s->tile_y);
+  s->tiles_y = (L.ny + rows - 1) / rows;
+  const long long tiles = (long long)s->tiles_x * s->tiles_y;
+  const int cz_min = s->own_chunk || !s->auto_chunk() ? s->chunk_z : kMinChunk;
+  if (tiles * ((L.nz + cz_min - 1) / cz_min) >= (1LL << 31)) return TETM_E_ARG;
   if (s->work) {
     dev_free(s->work, s->stream);
     s->work = nullptr;
   }
-  int* counts = nullptr;
-  CK(dev_alloc((void**)&counts, sizeof(int) * (size_t)items, s->stream));
-  item_counts<<<(unsigned)items, 256, 0, s->stream>>>(s->mask, L, s->tile_x, s->tile_y, s->chunk_z,
-                                                      s->tiles_x, s->tiles_y, (int)items, counts);
-  std::vector<int> h((size_t)items);
+  const size_t n = (size_t)tiles * L.nz;
+  uint8_t* act = nullptr;
+  CK(dev_alloc((void**)&act, n, s->stream));
+  tile_activity<<<(unsigned)std::min<size_t>((n + 7) / 8, 1u << 16), 256, 0, s->stream>>>(
+      s->mask, L, s->tile_x, rows, s->tiles_x, (long long)n, act);
+  s->act.resize(n);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), counts, sizeof(int) * (size_t)items,
-                                            cudaMemcpyDeviceToHost, s->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(s->act.data(), act, n, cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  dev_free(counts, s->stream);
+  dev_free(act, s->stream);
   if (e != cudaSuccess) return cuda_fail(e);
-  // the items that own a field-carrying cell, in grid order: items that run
-  // at the same time are neighbours and share their halo rows through L2
-  // (ordering the list by work instead was measured 1.3x slower)
+  if (!s->own_chunk) s->chunk_z = s->auto_chunk() ? choose_chunk(s, 1) : kChunk;
+  s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
   std::vector<int> list;
-  list.reserve((size_t)items);
-  for (long long q = 0; q < items; ++q)
-    if (h[(size_t)q]) list.push_back((int)q);
+  work_list(s, s->chunk_z, &list);
   s->n_work = (int)list.size();
   s->work_host = list;
   if (3 * s->n_work > s->diag.cap) {  // balance reductions keep three partials per work item
@@ -402,6 +454,7 @@ StepArgs<T> tetm::step_args(tetm_solver* s, bool fused) {
     a.co.u[c] = (T)(((c == kEZ || c == kHZ) ? 2.0 * s->alpha : s->alpha) * s->minv_c[c]);
     a.co.ua[c] = (const T*)s->ua[c];
   }
+  a.cstep = (unsigned)(field_step(s->L, s->esz) / 16);
   a.co.mask = s->mask;
   a.L = s->L;
   a.n = s->step;
@@ -452,7 +505,7 @@ WorkView work_view(const tetm_solver* s) {
   v.items = s->work;
   v.n_items = s->n_work;
   v.tile_x = s->tile_x;
-  v.tile_y = s->tile_y;
+  v.tile_y = slab_rows(s->tile_x, s->tile_y);
   v.chunk_z = s->chunk_z;
   v.tiles_x = s->tiles_x;
   v.tiles_y = s->tiles_y;
@@ -627,8 +680,7 @@ int set_fields_t(tetm_solver* s, int comp, const double* host) {
 // releases every device array of the solve, in the order of its stream
 void free_all(tetm_solver* s) {
   cudaStream_t st = s->stream;
-  for (int b = 0; b < 2; ++b)
-    for (int c = 0; c < 6; ++c) dev_free(s->set[b][c], st);
+  for (int b = 0; b < 2; ++b) dev_free(s->set[b][0], st);
   for (int c = 0; c < 6; ++c) {
     dev_free(s->minv_a[c], st);
     dev_free(s->m_a[c], st);
@@ -723,18 +775,20 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   s->kernel = TETM_KERNEL_FUSED;
   s->uniform = uniform;
   s->vacuum = uniform && eps_u == 1.0 && mu_u == 1.0;
-  // float32: the slab kernel (kernels_slab.cu; 56 x 12 tiles with
-  // coefficient arrays); float64: the warp-tiled kernel (kernels_warp.cu)
+  // float32: the slab kernel (kernels_slab.cu; named 56 x 12 with
+  // coefficient arrays); float64: the band kernels (kernels_band.cu), the
+  // warp-tiled kernel (kernels_warp.cu) once a shape is set
   s->tile_x = s->esz == 4 ? 56 : 28;
   s->tile_y = s->esz == 4 ? (uniform ? 28 : 12) : 20;
-  s->chunk_z = 32;
+  s->chunk_z = kChunk;
   int rc = TETM_OK;
-  const size_t fbytes = (size_t)s->L.count * s->esz;
-  for (int b = 0; b < 2 && rc == TETM_OK; ++b)
-    for (int c = 0; c < 6 && rc == TETM_OK; ++c) {
-      rc = dalloc(s, &s->set[b][c], fbytes);
-      if (rc == TETM_OK) rc = cudaMemsetAsync(s->set[b][c], 0, fbytes, s->stream) == cudaSuccess ? TETM_OK : TETM_E_CUDA;
-    }
+  const size_t fstep = field_step(s->L, s->esz), fbytes = 5 * fstep + (size_t)s->L.count * s->esz;
+  for (int b = 0; b < 2 && rc == TETM_OK; ++b) {
+    rc = dalloc(s, &s->set[b][0], fbytes);
+    if (rc != TETM_OK) break;
+    for (int c = 1; c < 6; ++c) s->set[b][c] = (char*)s->set[b][0] + c * fstep;
+    rc = cudaMemsetAsync(s->set[b][0], 0, fbytes, s->stream) == cudaSuccess ? TETM_OK : TETM_E_CUDA;
+  }
   if (rc == TETM_OK) rc = dalloc(s, (void**)&s->mask, (size_t)s->L.count);
   if (rc == TETM_OK) rc = cudaMemsetAsync(s->mask, 0, (size_t)s->L.count, s->stream) == cudaSuccess ? TETM_OK : TETM_E_CUDA;
   if (rc == TETM_OK) rc = dalloc(s, (void**)&s->diag.part, sizeof(double) * 2048);
@@ -928,6 +982,7 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   if (s->scheme == TETM_SCHEME_YEE) {  // Yee's fused kernel has one tile shape
     if (tx != s->tile_x || ty != s->tile_y) return TETM_E_UNSUPPORTED;
     if (cz < 4) return TETM_E_ARG;
+    if (chunk_z) s->own_chunk = true;
     s->chunk_z = cz;
     return rebuild_work(s);
   }
@@ -935,7 +990,7 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   if ((!fused_shape_ok(tx, ty) && !warp_shape_ok(tx, ty) && !slab_u && !slab_m) || cz < 4)
     return TETM_E_ARG;
   // per-entry coefficients (general materials) run on the warp-tiled kernel
-  // and on the slab kernel's 56 x 12 tiles; one material on its 56 x 28 tiles
+  // and on the slab kernel as 56 x 12; one material there as 56 x 28
   if (!s->uniform && tx != 28 && !slab_m && s->kernel == TETM_KERNEL_FUSED)
     return TETM_E_UNSUPPORTED;
   if (s->uniform && slab_m && !slab_u) return TETM_E_UNSUPPORTED;
@@ -943,6 +998,7 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   if ((slab_u || slab_m) && s->esz != 4) return TETM_E_UNSUPPORTED;
   if (s->kernel == TETM_KERNEL_TWOSTEP && !fused2_shape_ok(tx, ty)) return TETM_E_UNSUPPORTED;
   if (tile_x || tile_y || chunk_z) s->own_shape = true;
+  if (chunk_z) s->own_chunk = true;
   if (tx == s->tile_x && ty == s->tile_y && cz == s->chunk_z && s->work) return TETM_OK;
   s->tile_x = tx;
   s->tile_y = ty;
@@ -1254,7 +1310,7 @@ int tetm_get_info(tetm_solver* s, tetm_info* info) {
   info->step = s->step;
   info->device_bytes = s->device_bytes;
   info->active_cells = s->active_cells;
-  info->processed_cells = (long long)s->n_work * s->tile_x * s->tile_y * s->chunk_z;
+  info->processed_cells = (long long)s->n_work * s->tile_x * slab_rows(s->tile_x, s->tile_y) * s->chunk_z;
   info->kernel = s->kernel;
   info->precision = s->g.precision;
   info->tile_x = s->tile_x;

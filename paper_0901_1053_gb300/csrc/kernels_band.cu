@@ -151,10 +151,8 @@ __global__ void __launch_bounds__(kBThreads, 4) band_tm(const StepArgs<double> a
       e = ez[id] + coef<MAT>(a, kEZ, it.base + id) * cur;                           // U3
       if (t.r < R && t.c < W) {
         a.out[kEZ][it.base + id] = e;
-        if (line) {  // one item owns the line's node of a plane: one sample a step, no atomics
-          const long long mm = (a.n + a.b.kshift) - it.k - a.b.c0;
-          if (mm >= a.b.m_min && mm <= a.b.m_max) a.b.W[mm - a.b.m_min] -= e * a.b.inv_q;
-        }
+        // one item owns the line's node of a plane: a sample gets one addition a step
+        if (line) add_wake(a.b, (a.n + a.b.kshift) - it.k - a.b.c0, e);
       }
     }
     ezn[t.r * wx + t.c] = e;

@@ -778,7 +778,7 @@ __global__ void balance_pass2(const double* part_w, const double* part_e, const 
 }
 
 // threads per item: whole warps splitting the tile's columns evenly (224 for
-// a 56 x 28 tile)
+// 56 x 12 nodes)
 int balance_threads(const WorkView& wv) {
   const int area = wv.tile_x * wv.tile_y;
   const int rounds = (area + 255) / 256;

@@ -1,15 +1,28 @@
 // Block-tiled fused step, float32 (Sec. 4.2, Eq. (23)).
 //
-// One CTA of 512 threads per SM takes (tile, z chunk) work items in turn. A
-// tile owns 56 x 28 nodes and loads 64 x 32 (4 halo columns and 2 halo rows on
-// each side: the ten updates reach two nodes sideways); with coefficient
-// arrays two CTAs of 256 threads per SM do the same on 56 x 12 tiles (64 x 16
-// loaded), one CTA's barriers and copy waits overlapping the other's work.
-// Thread t holds the four consecutive columns 4 (t mod 16) .. +3 of row
-// t / 16 (a quad), so its loads and stores are 16-byte vectors, and marches
-// through the chunk plane by plane with the z-state of its quad in registers
-// (old e_x, e_y, new h_x, h_y of the planes below): no per-row state in
-// shared memory.
+// Two CTAs of 256 threads per SM take (tile, z chunk) work items in turn. A
+// tile owns 56 x 12 nodes and loads 64 x 16 (4 halo columns and 2 halo rows on
+// each side: the ten updates reach two nodes sideways), so one CTA's barriers
+// and copy waits overlap the other's work. Thread t holds the four consecutive
+// columns 4 (t mod 16) .. +3 of row t / 16 (a quad), so its loads and stores
+// are 16-byte vectors, and marches through the chunk plane by plane with the
+// z-state of its quad in registers (old e_x, e_y, new h_x, h_y of the planes
+// below): no per-row state in shared memory.
+//
+// What bounds it: the shared-memory and load/store pipe together with the
+// latency of the next plane's loads, not DRAM. With one material on 256 x 256
+// x 2048 a step takes 395 us, of which the arithmetic and barriers alone take
+// 209 us, and all inputs from L2 instead of DRAM 373 us. Tried on the way (us
+// per step on 256 x 256 x 1024 / 2048 and on a 16-solve batch's longest
+// solve): one CTA of 512 threads on 64 x 32 boxes in scalar arithmetic 225 /
+// 402 / 534; the same with packed pairs of float32 (half the issue slots for
+// the same roundings) 210 / 394 / 582; 64 x 16 boxes in two CTAs, packed, 204 /
+// 395 / 476 and 32.8 instead of 54.7 on 48 x 48 x 192, where a grid of few
+// tiles makes 2.3 times the items. The rows loaded in vain (4 of 16 instead of
+// 4 of 32) cost less than the waits of a lone CTA. A ring for all six inputs
+// instead of register loads, and tensor-map copies into it, were slower (the
+// ring's reads go through the pipe that is full), and so were later loads of
+// e_x, e_y (238 us) and a sweep unrolled by three planes (264 us: code size).
 //
 // Only entries that carry a field move through the per-thread loads and
 // stores. Each thread reads the activity bytes of its quad (one 32-bit word
@@ -58,14 +71,11 @@ namespace tetm {
 
 namespace {
 
-constexpr int kSX = 64, kSY = 32;   // loaded columns, rows
-constexpr int kOX = 56, kOY = 28;   // owned columns, rows
-constexpr int kQ = kSX / 4;         // column quads per row
-constexpr int kSThreads = kQ * kSY; // 512
-// with coefficient arrays: a 64 x 16 box (56 x 12 owned), two CTAs of 256
-// threads per SM, whose barriers interleave
-constexpr int kSYM = 16, kOYM = 12;
-constexpr int kMThreads = kQ * kSYM; // 256
+constexpr int kSX = 64, kSY = 16;    // loaded columns, rows
+constexpr int kOX = 56, kOY = 12;    // owned columns, rows
+constexpr int kQ = kSX / 4;          // column quads per row
+constexpr int kSThreads = kQ * kSY;  // 256
+constexpr int kNamedY = 28;          // tetm_set_tiling names the one-material shape 56 x 28, the other 56 x 12
 
 // One material: a two-plane ring of e_z and h_z (one coefficient per
 // component, switched by the activity bytes) and two exchange buffers, laid
@@ -86,7 +96,7 @@ struct SlabSmemU {
 // exchange buffers of the skewed sweep (hx~, ez', ex~, hz'), 160 KB, in one
 // array with a spare row at the end (reads past a buffer's edge stay inside).
 struct SlabSmemM {
-  static constexpr int kP = kSYM * kSX;
+  static constexpr int kP = kSY * kSX;
   float f[20 * kP + kSX];  // e_z slots (2), h_z slots (2), 2 x 6 coefficient planes, x1..x4, spare row
   int next[2];
   __device__ __forceinline__ float* ez(int s) { return f + s * kP; }
@@ -147,23 +157,98 @@ __device__ __forceinline__ void sts4(float* p, const Q4& a) {
   *reinterpret_cast<float4*>(p) = make_float4(a.v[0], a.v[1], a.v[2], a.v[3]);
 }
 
+// Pairs of float32 in 64-bit registers: one packed instruction rounds each
+// half as the scalar one does. A quad is two pairs.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float lo(f2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi(f2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+struct P4 {
+  f2 a, b;  // columns 0, 1 and 2, 3
+};
+__device__ __forceinline__ P4 fma4(const P4& c, const P4& x, const P4& y) {
+  P4 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.a) : "l"(c.a), "l"(x.a), "l"(y.a));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.b) : "l"(c.b), "l"(x.b), "l"(y.b));
+  return r;
+}
+__device__ __forceinline__ P4 sub4(const P4& x, const P4& y) {
+  P4 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.a) : "l"(x.a), "l"(y.a));
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(x.b), "l"(y.b));
+  return r;
+}
+// 16-byte accesses straight from and to register pairs
+__device__ __forceinline__ P4 ldp(const float* p) {
+  P4 r;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(r.a), "=l"(r.b) : "r"(su32(p)) : "memory");
+  return r;
+}
+__device__ __forceinline__ void stp(float* p, const P4& v) {
+  asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(su32(p)), "l"(v.a), "l"(v.b) : "memory");
+}
+__device__ __forceinline__ P4 ldg_if(const float* p, unsigned c) {
+  P4 r;
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n mov.b64 %0, 0;\n mov.b64 %1, 0;\n"
+      " @q ld.global.nc.v2.b64 {%0, %1}, [%2];\n}"
+      : "=l"(r.a), "=l"(r.b)
+      : "l"(p), "r"(c));
+  return r;
+}
+__device__ __forceinline__ void stg_if(float* p, const P4& v, unsigned c) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q st.global.v2.b64 [%0], {%1, %2};\n}" ::"l"(p),
+               "l"(v.a), "l"(v.b), "r"(c)
+               : "memory");
+}
+
 // the neighbouring quad's value one column left (x-1) or right (x+1) of this
 // quad (lanes: one row per half warp); at the tile edge a lane takes a value
 // of the other half warp's row, which only halo nodes read
 __device__ __forceinline__ float left_any(float v3) { return __shfl_up_sync(0xffffffffu, v3, 1); }
 __device__ __forceinline__ float right_any(float v0) { return __shfl_down_sync(0xffffffffu, v0, 1); }
 
+// the quad one column on minus the quad, and the quad one column back minus it
+// (an exchanged column more: see slab_item)
+__device__ __forceinline__ P4 diff_right(const P4& v) {
+  const float r = right_any(lo(v.a));
+  return P4{pk(hi(v.a) - lo(v.a), lo(v.b) - hi(v.a)), pk(hi(v.b) - lo(v.b), r - hi(v.b))};
+}
+__device__ __forceinline__ P4 diff_left(const P4& v) {
+  const float l = left_any(hi(v.b));
+  return P4{pk(l - lo(v.a), lo(v.a) - hi(v.a)), pk(hi(v.a) - lo(v.b), lo(v.b) - hi(v.b))};
+}
+
 // One (tile, z-chunk) work item of solve a with one material (the ten
 // updates of every plane of the chunk, plane by plane: four block barriers
-// per plane).
+// per plane). SHARED: a lies in shared memory (batches) instead of the
+// parameter space. There each array's address is its set's pointer, kept in
+// registers, plus a multiple of cstep: read from shared memory the twelve
+// pointers took a slot each of the pipe that bounds the sweep in every plane
+// (batch of 16 solves: 558 us per step of the longest, so 476). From the
+// parameter space the twelve pointers are free, and one running pointer per
+// set was measured 1.7 times slower.
 //
-// The reads of a neighbour one row or column outside the 64 x 32 box take
+// The reads of a neighbour one row or column outside the 64 x 16 box take
 // whatever the neighbouring shared-memory words or lanes hold, without an
 // edge test. Each of the six stages reaches one node sideways, and a value
 // computed from an outside neighbour is wrong only on the box's outermost
 // row or column; through the stages that error reaches at most two rows and
-// two columns in, all of them halo (the tile owns rows 2..29 and columns
+// two columns in, all of them halo (the tile owns rows 2..13 and columns
 // 4..59 of the box), and halo nodes are never stored.
+template <bool SHARED>
 __device__ __forceinline__ void slab_item(const StepArgs<float>& a, int item, SlabSmemU& S) {
   constexpr int kSD = SlabSmemU::SD;
   const int tid = threadIdx.x, q = tid % kQ, row = tid / kQ;
@@ -172,7 +257,23 @@ __device__ __forceinline__ void slab_item(const StepArgs<float>& a, int item, Sl
   const float uEX = a.co.u[kEX], uEY = a.co.u[kEY], uEZ = a.co.u[kEZ];
   const float uHX = a.co.u[kHX], uHY = a.co.u[kHY], uHZ = a.co.u[kHZ];
   const int ntile = a.tiles_x * a.tiles_y;
-  const Q4 zero{{0.f, 0.f, 0.f, 0.f}};
+  const P4 zero{0ull, 0ull};
+  const float* const in0 = a.in[0];
+  float* const out0 = a.out[0];
+  const uint8_t* const mask = a.co.mask;
+  const unsigned cs = a.cstep;
+  auto in_of = [&](int c) -> const float* {
+    if constexpr (SHARED)
+      return reinterpret_cast<const float*>(reinterpret_cast<const char*>(in0) + (unsigned long long)cs * (16u * c));
+    else
+      return a.in[c];
+  };
+  auto out_of = [&](int c) -> float* {
+    if constexpr (SHARED)
+      return reinterpret_cast<float*>(reinterpret_cast<char*>(out0) + (unsigned long long)cs * (16u * c));
+    else
+      return a.out[c];
+  };
   const int tile = item % ntile, chunk = item / ntile;
   const int gx0 = (tile % a.tiles_x) * kOX - 4;  // global i of loaded column 0
   const int gy0 = (tile / a.tiles_x) * kOY - 2;  // global j of loaded row 0
@@ -190,8 +291,8 @@ __device__ __forceinline__ void slab_item(const StepArgs<float>& a, int item, Sl
   const long long qoff = (long long)(gj + 2) * PX + cx + 4 * q;
   const bool own_q = q >= 1 && q <= kQ - 2 && row >= 2 && row < kSY - 2 && gj < L.ny;
   auto gidx = [&](int k) { return (long long)(k + 1) * SZ + qoff; };
-  auto word = [&](int k) -> unsigned { return ld_word_if(a.co.mask + gidx(k), inq); };
-  auto load_if = [&](const float* base, int k, unsigned p) -> Q4 { return ld4_if(base + gidx(k), p); };
+  auto word = [&](int k) -> unsigned { return ld_word_if(mask + gidx(k), inq); };
+  auto load_if = [&](const float* base, int k, unsigned p) -> P4 { return ldg_if(base + gidx(k), p); };
   // plane k into its slot: each thread copies the quad of its own node row
   // and columns of e_z, h_z, only where one of the quad's nodes carries that
   // component (zeros otherwise: the entry holds zero), so the ring reads no
@@ -200,8 +301,8 @@ __device__ __forceinline__ void slab_item(const StepArgs<float>& a, int item, Sl
   auto issue_q = [&](int k, unsigned mw) {
     const int s = (k - kstart) % kSD;
     const long long g = inq ? gidx(k) : 0;
-    cp16_or_zero(S.ez(s) + row * kSX + 4 * q, a.in[kEZ] + g, has(mw, kEZ));
-    cp16_or_zero(S.hz(s) + row * kSX + 4 * q, a.in[kHZ] + g, has(mw, kHZ));
+    cp16_or_zero(S.ez(s) + row * kSX + 4 * q, in_of(kEZ) + g, has(mw, kEZ));
+    cp16_or_zero(S.hz(s) + row * kSX + 4 * q, in_of(kHZ) + g, has(mw, kHZ));
   };
   // activity words of planes k .. k + kSD (m[0] of the plane being worked
   // on; m[kSD] of the plane whose copy is issued next); z-state and the
@@ -216,146 +317,93 @@ __device__ __forceinline__ void slab_item(const StepArgs<float>& a, int item, Sl
   }
   cp_wait<kSD - 1>();
   __syncthreads();  // plane kstart's slot is in
-  Q4 ex0 = load_if(a.in[kEX], kstart, hw(m[0], kEX)), ey0 = load_if(a.in[kEY], kstart, hw(m[0], kEY));
-  Q4 hxc = load_if(a.in[kHX], kstart, hw(m[0], kHX)), hyc = load_if(a.in[kHY], kstart, hw(m[0], kHY));
-  Q4 ex1 = load_if(a.in[kEX], kstart + 1, hw(m[1], kEX)), ey1 = load_if(a.in[kEY], kstart + 1, hw(m[1], kEY));
-  Q4 hxp = zero, hyp = zero;
+  P4 ex0 = load_if(in_of(kEX), kstart, hw(m[0], kEX)), ey0 = load_if(in_of(kEY), kstart, hw(m[0], kEY));
+  P4 hxc = load_if(in_of(kHX), kstart, hw(m[0], kHX)), hyc = load_if(in_of(kHY), kstart, hw(m[0], kHY));
+  P4 ex1 = load_if(in_of(kEX), kstart + 1, hw(m[1], kEX)), ey1 = load_if(in_of(kEY), kstart + 1, hw(m[1], kEY));
+  P4 hxp = zero, hyp = zero;
   const bool line_row = a.b.on && gj == a.b.j0;
   const bool line_q = line_row && a.b.i0 >= gi && a.b.i0 < gi + 4;  // the quad holds the bunch line node
 
   for (int k = kstart; k < k1; ++k) {
     const int s = (k - kstart) % kSD;
     // next plane's register inputs and the activity word kSD + 1 planes on, early
-    Q4 hxn_in, hyn_in, exn_in, eyn_in;
+    P4 hxn_in, hyn_in, exn_in, eyn_in;
     unsigned mn = 0u;
     const bool more = k + 1 < k1;
     if (more) {
-      hxn_in = load_if(a.in[kHX], k + 1, hw(m[1], kHX));
-      hyn_in = load_if(a.in[kHY], k + 1, hw(m[1], kHY));
-      exn_in = load_if(a.in[kEX], k + 2, hw(m[2], kEX));
-      eyn_in = load_if(a.in[kEY], k + 2, hw(m[2], kEY));
+      hxn_in = load_if(in_of(kHX), k + 1, hw(m[1], kHX));
+      hyn_in = load_if(in_of(kHY), k + 1, hw(m[1], kHY));
+      exn_in = load_if(in_of(kEX), k + 2, hw(m[2], kEX));
+      eyn_in = load_if(in_of(kEY), k + 2, hw(m[2], kEY));
       if (k + kSD + 1 <= k1) mn = word(k + kSD + 1);
     }
     // slot inputs: e_z, h_z of this quad and its neighbours
     const float* sez = S.ez(s) + row * kSX + 4 * q;
     const float* shz = S.hz(s) + row * kSX + 4 * q;
-    const Q4 ez = lds4(sez);
-    const Q4 ezU = lds4(sez + kSX);
-    const float ezR = sez[4];
-    const Q4 hz = lds4(shz);
-    const Q4 hzD = lds4(shz - kSX);
-    const float hzL = shz[-1];
+    const P4 ez = ldp(sez);
+    const P4 ezU = ldp(sez + kSX);
+    const P4 hz = ldp(shz);
+    const P4 hzD = ldp(shz - kSX);
     float* const x1 = S.x1() + row * kSX + 4 * q;  // this thread's quad in the exchange buffers
     float* const x2 = S.x2() + row * kSX + 4 * q;
     // one coefficient per component, switched by the activity bytes
-    float cHX[4], cHY[4], cEZ[4], cEX[4], cEY[4], cHZ[4], dey[4], dex[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const unsigned b = (m[0] >> (8 * e)) & 0xFFu;
-      cEX[e] = (b & 1) ? uEX : 0.f;
-      cEY[e] = (b & 2) ? uEY : 0.f;
-      cEZ[e] = (b & 4) ? uEZ : 0.f;
-      cHX[e] = (b & 8) ? uHX : 0.f;
-      cHY[e] = (b & 16) ? uHY : 0.f;
-      cHZ[e] = (b & 32) ? uHZ : 0.f;
-    }
-    Q4 hxa, hya;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      dey[e] = ey1.v[e] - ey0.v[e];
-      dex[e] = ex1.v[e] - ex0.v[e];
-      const float ezx = e < 3 ? ez.v[e + 1] : ezR;
-      hxa.v[e] = hxc.v[e] + cHX[e] * (dey[e] - (ezU.v[e] - ez.v[e]));   // U1
-      hya.v[e] = hyc.v[e] + cHY[e] * (-dex[e] + (ezx - ez.v[e]));      // U2
-    }
-    sts4(x1, hxa);
+    const unsigned w = m[0];
+    auto co = [&](int c, float u) {
+      auto at = [&](int e) { return (w & (1u << (8 * e + c))) ? u : 0.f; };
+      return P4{pk(at(0), at(1)), pk(at(2), at(3))};
+    };
+    const P4 cHX = co(kHX, uHX), cHY = co(kHY, uHY), cEZ = co(kEZ, uEZ);
+    const P4 cEX = co(kEX, uEX), cEY = co(kEY, uEY), cHZ = co(kHZ, uHZ);
+    const P4 dey = sub4(ey1, ey0), dex = sub4(ex1, ex0);
+    const P4 hxa = fma4(cHX, sub4(dey, sub4(ezU, ez)), hxc);        // U1
+    const P4 hya = fma4(cHY, sub4(diff_right(ez), dex), hyc);       // U2
+    stp(x1, hxa);
     __syncthreads();  // (1) the slot is read and hx~ is out
     if (k + kSD < k1) issue_q(k + kSD, m[kSD]);  // into the freed slot
     cp_commit();
     // S2: ez' = ez + 2a M^-1 (P_y^T hx~ - P_x^T hy~ - jj_z)
-    const Q4 hxaD = lds4(x1 - kSX);
-    const float hyaL = left_any(hya.v[3]);
-    float cur[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float hyl = e > 0 ? hya.v[e - 1] : hyaL;
-      cur[e] = (hxaD.v[e] - hxa.v[e]) - (hyl - hya.v[e]);
-    }
+    P4 cur = sub4(sub4(ldp(x1 - kSX), hxa), diff_left(hya));
     if (line_q) {  // the bunch current on its line (one quad of a tile row)
       const long long dd = (long long)k - (a.n + a.b.kshift) + a.b.c0;
       if (dd >= -a.b.c0 && dd < a.b.c0) {
         const float jj = a.b.J[dd + a.b.c0];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (gi + e == a.b.i0) cur[e] -= jj;
+        const int e = a.b.i0 - gi;
+        cur = sub4(cur, P4{pk(e == 0 ? jj : 0.f, e == 1 ? jj : 0.f), pk(e == 2 ? jj : 0.f, e == 3 ? jj : 0.f)});
       }
     }
-    Q4 ezn;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) ezn.v[e] = ez.v[e] + cEZ[e] * cur[e];   // U3
-    sts4(x2, ezn);
+    const P4 ezn = fma4(cEZ, cur, ez);                              // U3
+    stp(x2, ezn);
     __syncthreads();  // (2)
     // S3: hx', hy'
-    const Q4 eznU = lds4(x2 + kSX);
-    const float eznR = right_any(ezn.v[0]);
-    Q4 hxn, hyn;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float ezx = e < 3 ? ezn.v[e + 1] : eznR;
-      hxn.v[e] = hxa.v[e] + cHX[e] * (dey[e] - (eznU.v[e] - ezn.v[e]));  // U4
-      hyn.v[e] = hya.v[e] + cHY[e] * (-dex[e] + (ezx - ezn.v[e]));     // U5
-    }
+    const P4 hxn = fma4(cHX, sub4(dey, sub4(ldp(x2 + kSX), ezn)), hxa);  // U4
+    const P4 hyn = fma4(cHY, sub4(diff_right(ezn), dex), hya);           // U5
     const bool st = k >= k0 && own_q;
     const unsigned ms = st ? m[0] : 0u;  // the plane's word where this thread stores
-    st4_if(a.out[kEZ] + gidx(k), ezn, hw(ms, kEZ));
-    st4_if(a.out[kHX] + gidx(k), hxn, hw(ms, kHX));
-    st4_if(a.out[kHY] + gidx(k), hyn, hw(ms, kHY));
-    if (st) {
-      if (line_q && a.b.i0 < L.nx) {
-        const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-        if (mm >= a.b.m_min && mm <= a.b.m_max)
-        {
-          const int e = a.b.i0 - gi;  // the quad's entry on the bunch line (no indexed register array)
-          const float v = e == 0 ? ezn.v[0] : e == 1 ? ezn.v[1] : e == 2 ? ezn.v[2] : ezn.v[3];
-          a.b.W[mm - a.b.m_min] -= (double)v * a.b.inv_q;
-        }
-      }
+    stg_if(out_of(kEZ) + gidx(k), ezn, hw(ms, kEZ));
+    stg_if(out_of(kHX) + gidx(k), hxn, hw(ms, kHX));
+    stg_if(out_of(kHY) + gidx(k), hyn, hw(ms, kHY));
+    if (st && line_q && a.b.i0 < L.nx) {
+      const int e = a.b.i0 - gi;  // the quad's entry on the bunch line (no indexed register array)
+      add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0,
+               e == 0 ? lo(ezn.a) : e == 1 ? hi(ezn.a) : e == 2 ? lo(ezn.b) : hi(ezn.b));
     }
     // S4: ex~, ey~ with the new hx, hy of this plane and of the plane below
-    Q4 exa, eya;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float hzl = e > 0 ? hz.v[e - 1] : hzL;
-      exa.v[e] = ex0.v[e] + cEX[e] * ((hyp.v[e] - hyn.v[e]) - (hzD.v[e] - hz.v[e]));   // U6
-      eya.v[e] = ey0.v[e] + cEY[e] * (-(hxp.v[e] - hxn.v[e]) + (hzl - hz.v[e]));       // U7
-    }
-    sts4(x1, exa);
+    const P4 dhy = sub4(hyp, hyn), dhx = sub4(hxp, hxn);
+    const P4 exa = fma4(cEX, sub4(dhy, sub4(hzD, hz)), ex0);        // U6
+    const P4 eya = fma4(cEY, sub4(diff_left(hz), dhx), ey0);        // U7
+    stp(x1, exa);
     __syncthreads();  // (3)
     // S5: hz'
-    const Q4 exaU = lds4(x1 + kSX);
-    const float eyaR = right_any(eya.v[0]);
-    Q4 hzn;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float eyx = e < 3 ? eya.v[e + 1] : eyaR;
-      hzn.v[e] = hz.v[e] + cHZ[e] * ((exaU.v[e] - exa.v[e]) - (eyx - eya.v[e]));      // U8
-    }
-    sts4(x2, hzn);
+    const P4 hzn = fma4(cHZ, sub4(sub4(ldp(x1 + kSX), exa), diff_right(eya)), hz);  // U8
+    stp(x2, hzn);
     cp_wait<kSD - 1>();  // this thread's copies of the next plane are in
     __syncthreads();  // (4) (and the next plane's slot is in)
     // S6: ex', ey'
-    const Q4 hznD = lds4(x2 - kSX);
-    const float hznL = left_any(hzn.v[3]);
-    Q4 exn, eyn;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float hzl = e > 0 ? hzn.v[e - 1] : hznL;
-      exn.v[e] = exa.v[e] + cEX[e] * ((hyp.v[e] - hyn.v[e]) - (hznD.v[e] - hzn.v[e]));   // U9
-      eyn.v[e] = eya.v[e] + cEY[e] * (-(hxp.v[e] - hxn.v[e]) + (hzl - hzn.v[e]));       // U10
-    }
-    st4_if(a.out[kEX] + gidx(k), exn, hw(ms, kEX));
-    st4_if(a.out[kEY] + gidx(k), eyn, hw(ms, kEY));
-    st4_if(a.out[kHZ] + gidx(k), hzn, hw(ms, kHZ));
+    const P4 exn = fma4(cEX, sub4(dhy, sub4(ldp(x2 - kSX), hzn)), exa);  // U9
+    const P4 eyn = fma4(cEY, sub4(diff_left(hzn), dhx), eya);            // U10
+    stg_if(out_of(kEX) + gidx(k), exn, hw(ms, kEX));
+    stg_if(out_of(kEY) + gidx(k), eyn, hw(ms, kEY));
+    stg_if(out_of(kHZ) + gidx(k), hzn, hw(ms, kHZ));
     // carry the z-state, take the prefetched inputs
     hxp = hxn;
     hyp = hyn;
@@ -389,7 +437,7 @@ __device__ __forceinline__ void slab_item_mat(const StepArgs<float>& a, int item
   const Q4 zero{{0.f, 0.f, 0.f, 0.f}};
   const int tile = item % ntile, chunk = item / ntile;
   const int gx0 = (tile % a.tiles_x) * kOX - 4;  // global i of loaded column 0
-  const int gy0 = (tile / a.tiles_x) * kOYM - 2;  // global j of loaded row 0
+  const int gy0 = (tile / a.tiles_x) * kOY - 2;  // global j of loaded row 0
   const int k0 = chunk * a.chunk_z, k1 = min(k0 + a.chunk_z, L.nz);
   const int kstart = k0 - 1;                   // the plane below the chunk: its new h_x, h_y feed U6, U7 of k0
   const int cx = gx0 + L.ox;                   // layout column of loaded column 0
@@ -401,7 +449,7 @@ __device__ __forceinline__ void slab_item_mat(const StepArgs<float>& a, int item
   const int gi = gx0 + 4 * q, gj = gy0 + row;
   const bool inq = gj + 2 < L.ny + 4 && cx + 4 * q + 4 <= PX;  // the quad lies inside the arrays
   const long long qoff = (long long)(gj + 2) * PX + cx + 4 * q;
-  const bool own_q = q >= 1 && q <= kQ - 2 && row >= 2 && row < kSYM - 2 && gj < L.ny;
+  const bool own_q = q >= 1 && q <= kQ - 2 && row >= 2 && row < kSY - 2 && gj < L.ny;
   const int qo = row * kSX + 4 * q;  // this thread's quad in a box plane
   float* const x1 = S.x(1) + qo;     // and in the exchange buffers
   float* const x2 = S.x(2) + qo;
@@ -599,12 +647,9 @@ __device__ __forceinline__ void slab_item_mat(const StepArgs<float>& a, int item
       st4_if(a.out[kHX] + gidx(p), hxN, hw(ms, kHX));
       st4_if(a.out[kHY] + gidx(p), hyN, hw(ms, kHY));
       if (st && line_q && a.b.i0 < L.nx) {
-        const long long mm = (a.n + a.b.kshift) - p - a.b.c0;
-        if (mm >= a.b.m_min && mm <= a.b.m_max) {
-          const int e = a.b.i0 - gi;  // the quad's entry on the bunch line (no indexed register array)
-          const float v = e == 0 ? ezn2.v[0] : e == 1 ? ezn2.v[1] : e == 2 ? ezn2.v[2] : ezn2.v[3];
-          a.b.W[mm - a.b.m_min] -= (double)v * a.b.inv_q;
-        }
+        const int e = a.b.i0 - gi;  // the quad's entry on the bunch line (no indexed register array)
+        const float v = e == 0 ? ezn2.v[0] : e == 1 ? ezn2.v[1] : e == 2 ? ezn2.v[2] : ezn2.v[3];
+        add_wake(a.b, (a.n + a.b.kshift) - p - a.b.c0, v);
       }
     }
     if (te && wte) {
@@ -647,7 +692,7 @@ __device__ __forceinline__ void slab_item_mat(const StepArgs<float>& a, int item
 }
 
 template <bool MAT>
-__global__ void __launch_bounds__(MAT ? kMThreads : kSThreads, MAT ? 2 : 1)
+__global__ void __launch_bounds__(kSThreads, 2)
     fused_step_slab(const StepArgs<float> a, int* sched) {
   using Smem = SlabSmem<MAT>;
   extern __shared__ __align__(128) unsigned char slab_raw[];
@@ -667,7 +712,7 @@ __global__ void __launch_bounds__(MAT ? kMThreads : kSThreads, MAT ? 2 : 1)
     if constexpr (MAT)
       slab_item_mat(a, item, S);
     else
-      slab_item(a, item, S);
+      slab_item<false>(a, item, S);
     wi = sched ? S.next[par] : wi + G;
     par ^= 1;
   }
@@ -684,7 +729,7 @@ __global__ void __launch_bounds__(MAT ? kMThreads : kSThreads, MAT ? 2 : 1)
 // Batches: one launch steps every active member (one material, float32);
 // work = (member, item) pairs, the member's arguments from device memory,
 // copied into shared memory for each item.
-__global__ void __launch_bounds__(kSThreads, 1)
+__global__ void __launch_bounds__(kSThreads, 2)
 fused_step_slab_batch(const BatchMember<float>* __restrict__ members, const int2* __restrict__ work,
                       const int* __restrict__ n_work_p, int* sched) {
   using Smem = SlabSmem<false>;
@@ -701,17 +746,16 @@ fused_step_slab_batch(const BatchMember<float>* __restrict__ members, const int2
     const int2 w = work[wi];
     const BatchMember<float>& mb = members[w.x];
     if (mb.active) {
-      // the member's arguments into shared memory once per item: the sweep
-      // reads them at every plane, and from global memory (where the
-      // single-solve kernel has them in its parameter space) each of those
-      // reads was a load on the critical path (the batch ran 28% slower)
+      // the member's arguments into shared memory once per item: what the
+      // sweep reads again from global memory (where the single-solve kernel
+      // has its parameter space) is a load on the critical path
       {
         const unsigned* s4 = reinterpret_cast<const unsigned*>(&mb.a);
         unsigned* d4 = reinterpret_cast<unsigned*>(&sargs);
         for (int i = tid; i < (int)(sizeof(StepArgs<float>) / 4); i += kSThreads) d4[i] = s4[i];
       }
       __syncthreads();
-      slab_item(sargs, w.y, S);
+      slab_item<true>(sargs, w.y, S);
     } else {
       // an item of a member past its limit: no work, but the ticket thread 0
       // wrote above must be visible before every thread reads it (slab_item
@@ -732,7 +776,8 @@ fused_step_slab_batch(const BatchMember<float>* __restrict__ members, const int2
 
 }  // namespace
 
-bool slab_shape_ok(int tx, int ty, bool mat) { return tx == kOX && ty == (mat ? kOYM : kOY); }
+bool slab_shape_ok(int tx, int ty, bool mat) { return tx == kOX && ty == (mat ? kOY : kNamedY); }
+int slab_rows(int tx, int ty) { return tx == kOX && ty == kNamedY ? kOY : ty; }
 
 namespace {
 template <bool MAT>
@@ -752,8 +797,7 @@ cudaError_t launch_slab(const StepArgs<float>& a, int* sched, cudaStream_t st) {
   }
   const int items = a.work ? a.n_work : a.tiles_x * a.tiles_y * a.n_chunks;
   if (items <= 0) return cudaSuccess;
-  constexpr int threads = MAT ? kMThreads : kSThreads, per_sm = MAT ? 2 : 1;
-  fused_step_slab<MAT><<<std::min(items, per_sm * sms), threads, smem, st>>>(a, sched);
+  fused_step_slab<MAT><<<std::min(items, 2 * sms), kSThreads, smem, st>>>(a, sched);
   return cudaGetLastError();
 }
 }  // namespace
@@ -774,7 +818,7 @@ cudaError_t launch_fused_slab_batch(BatchMember<float>* members, int n_members, 
     }
   }
   if (n_bound > 0) {
-    fused_step_slab_batch<<<std::min(n_bound, sms), kSThreads, smem, st>>>(members, work, n_work, sched);
+    fused_step_slab_batch<<<std::min(n_bound, 2 * sms), kSThreads, smem, st>>>(members, work, n_work, sched);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -131,10 +131,7 @@ __global__ void ref_update(StepArgs<T> a) {
     }
     const T ezn = ez[id] + c * cur;
     F[kEZ][id] = ezn;
-    if (line) {  // wake sample: W(s_m) -= ez^{n+1/2}(k) / Q with m = n - k - c0
-      const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-      if (mm >= a.b.m_min && mm <= a.b.m_max) a.b.W[mm - a.b.m_min] -= (double)ezn * a.b.inv_q;
-    }
+    if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);  // W(s_m) -= ez^{n+1/2}(k) / Q, m = n - k - c0
   } else if (C == kEX) {  // U6 / U9: ex += a M^-1 (P_z^T hy - P_y^T hz)
     F[kEX][id] = ex[id] + c * ((hy[id - sz] - hy[id]) - (hz[id - sy] - hz[id]));
   } else if (C == kEY) {  // U7 / U10: ey += a M^-1 (-P_z^T hx + P_x^T hz)
@@ -229,10 +226,7 @@ fused_step(const StepArgs<T> a) {
         a.out[kHX][id] = hxn;
         a.out[kHY][id] = hyn;
         a.out[kEZ][id] = ezn;
-        if (line) {
-          const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-          if (mm >= a.b.m_min && mm <= a.b.m_max) a.b.W[mm - a.b.m_min] -= (double)ezn * a.b.inv_q;
-        }
+        if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
       }
       // ---- TE stage at plane k (time n -> n+1) ----
       const T cEX = (m & 1) ? uEX : T(0), cEY = (m & 2) ? uEY : T(0), cHZ = (m & 32) ? uHZ : T(0);
@@ -363,10 +357,7 @@ fused_step2(const StepArgs<T> a) {
     __syncthreads();
     const T hx1 = hxa + cHX * (dey - (sE[sy + 1][sx] - ez1));   // U4
     const T hy1 = hya + cHY * (-dex + (sE[sy][sx + 1] - ez1));  // U5
-    if (own && line && k >= k0 && k < k1) {
-      const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-      if (mm >= a.b.m_min && mm <= a.b.m_max) atomicAdd(a.b.W + (mm - a.b.m_min), -(double)ez1 * a.b.inv_q);
-    }
+    if (own && line && k >= k0 && k < k1) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ez1);
     T ex1 = T(0), ey1 = T(0), hz1 = T(0);
     if (k >= k0 - 1) {
       const T cEX = (m0 & 1) ? uEX : T(0), cEY = (m0 & 2) ? uEY : T(0), cHZ = (m0 & 32) ? uHZ : T(0);
@@ -415,11 +406,7 @@ fused_step2(const StepArgs<T> a) {
           a.out[kHX][idp] = hx2;
           a.out[kHY][idp] = hy2;
           a.out[kEZ][idp] = ez2;
-          if (line) {
-            const long long mm = (a.n + 1 + a.b.kshift) - p - a.b.c0;
-            if (mm >= a.b.m_min && mm <= a.b.m_max)
-              atomicAdd(a.b.W + (mm - a.b.m_min), -(double)ez2 * a.b.inv_q);
-          }
+          if (line) add_wake(a.b, (a.n + 1 + a.b.kshift) - p - a.b.c0, ez2);
         }
         const T cEX2 = (mp & 1) ? uEX : T(0), cEY2 = (mp & 2) ? uEY : T(0), cHZ2 = (mp & 32) ? uHZ : T(0);
         const T dhy2 = hy2p - hy2, dhx2 = hx2p - hx2;

@@ -203,11 +203,7 @@ __device__ __forceinline__ void fused_step_warp_item(const StepArgs<T>& a, int i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) {
-              const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-              if (mm >= a.b.m_min && mm <= a.b.m_max)
-                a.b.W[mm - a.b.m_min] -= (double)ezn * a.b.inv_q;
-            }
+            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }
@@ -465,11 +461,7 @@ __device__ __forceinline__ void fused_step_warp_reg_item(const StepArgs<T>& a, i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) {
-              const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-              if (mm >= a.b.m_min && mm <= a.b.m_max)
-                a.b.W[mm - a.b.m_min] -= (double)ezn * a.b.inv_q;
-            }
+            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }
@@ -748,11 +740,7 @@ __device__ __forceinline__ void fused_step_warp_mat_item(const StepArgs<T>& a, i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) {
-              const long long mm = (a.n + a.b.kshift) - k - a.b.c0;
-              if (mm >= a.b.m_min && mm <= a.b.m_max)
-                a.b.W[mm - a.b.m_min] -= (double)ezn * a.b.inv_q;
-            }
+            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }

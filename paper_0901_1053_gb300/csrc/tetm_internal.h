@@ -61,6 +61,15 @@ struct BunchDev {
   double* WY;
 };
 
+// Longitudinal wake sample m of the bunch line's new e_z: one fire-and-forget
+// addition. As a load, an addition and a store the round trip to memory
+// (about 0.7 us) held up the block that marches the line at every plane of the
+// wake window.
+template <typename T>
+__device__ __forceinline__ void add_wake(const BunchDev<T>& b, long long m, T ez) {
+  if (m >= b.m_min && m <= b.m_max) atomicAdd(b.W + (m - b.m_min), -__dmul_rn((double)ez, b.inv_q));
+}
+
 // Transverse wake samples of plane k (step n -> n+1): W_x from the old e_x
 // and the new h_y of the x-edge at the observer line, W_y from the old e_y
 // and the new h_x of the y-edge; sample m = n + kshift - k - c0 as for W.
@@ -90,6 +99,7 @@ template <typename T>
 struct StepArgs {
   const T* in[6];       // state y^n (fused: read only)
   T* out[6];            // fused: state y^{n+1}; reference: == in (updated in place)
+  unsigned cstep;       // from one component's array to the next, in 16-byte units (in and out alike)
   Coefs<T> co;
   Layout L;
   long long n;          // step index of the state being advanced
@@ -139,9 +149,12 @@ template <typename T>
 cudaError_t launch_batch_advance(BatchMember<T>* members, int n_members, cudaStream_t st);
 
 // ---- block-tiled float32 step with a shared-memory ring (kernels_slab.cu):
-// tile 56 x 28, one CTA of 512 threads per SM; with coefficient arrays (mat)
-// tile 56 x 12, two CTAs of 256 threads per SM ------------------------------
+// 56 x 12 nodes per item, two CTAs of 256 threads per SM; tetm_set_tiling
+// names the shape 56 x 28 for one material and 56 x 12 with coefficient arrays
+// (mat) ---------------------------------------------------------------------
 bool slab_shape_ok(int tile_x, int tile_y, bool mat);
+// rows a work item of shape tile_x x tile_y owns (12 for the slab kernel's)
+int slab_rows(int tile_x, int tile_y);
 // one step of every active member of a float32 batch on the slab kernel
 // (work = (member, item) pairs counted at n_work in device memory, at most
 // n_bound; sched as below), the transverse wakes, then the device-side
@@ -238,11 +251,14 @@ cudaError_t launch_bunch_charge(double q, double sigma, double dz, double zc, in
 }  // namespace tetm
 
 // The solve behind a tetm_solver* handle (host bookkeeping and device arrays).
+// bytes from one component's array to the next within a field set
+inline size_t field_step(const tetm::Layout& L, size_t esz) { return ((size_t)L.count * esz + 255) & ~(size_t)255; }
+
 struct tetm_solver {
   tetm_grid g;
   size_t esz;
   tetm::Layout L;
-  void* set[2][6];
+  void* set[2][6];  // each set one allocation, the components field_step() apart
   int cur;
   uint8_t* mask;
   double minv_c[6];
@@ -263,9 +279,13 @@ struct tetm_solver {
   int* work;
   int n_work;
   bool own_shape;              // the caller chose the work shape (tetm_set_tiling)
+  bool own_chunk;              // and its planes per item
+  std::vector<uint8_t> act;    // per tile and plane (tile-major): the tile owns an active cell there
   int4* band;                  // float64: work items of the band kernels (the default work shape)
   int n_band, band_smem;
   std::vector<int> work_host;  // host copy of the work list
+  // the slab kernel's shape: planes per item by choose_chunk unless set
+  bool auto_chunk() const { return esz == 4 && tetm::slab_shape_ok(tile_x, tile_y, !uniform); }
   bool in_batch;               // stepped by a tetm_batch
   bool work_dirty;
   // bunch
@@ -327,6 +347,11 @@ template <typename T>
 StepArgs<T> step_args(tetm_solver* s, bool fused);
 // (re)build the list of (tile, chunk) work items that own a field-carrying cell
 int rebuild_work(tetm_solver* s);
+constexpr int kChunk = 32, kMinChunk = 4, kMaxChunk = 64;  // planes per work item: set ones start at kMinChunk
+// the slab kernel's planes per item for one of `share` solves that step
+// together, and the items of chunks of cz planes (both from s->act)
+int choose_chunk(const tetm_solver* s, int share);
+void work_list(const tetm_solver* s, int cz, std::vector<int>* list);
 // Device memory of solves and batches comes from one stream-ordered pool per
 // device: allocation and release are queued on the given stream, so neither
 // waits for work queued on other streams (cudaFree waits for the whole
