@@ -261,7 +261,8 @@ int tetm_set_kernel(tetm_solver* s, int32_t kernel);
  * solve whose shape was never set steps in two launches, one per half of the
  * step, over bands of rows of every plane (not a z-slab, which runs the
  * warp-tiled kernel; the shape reported, 28 x 20 x 32, is then the one the
- * balances walk); the fields are the same bits on all of them. Any value
+ * balances walk), and so does a small float32 one of one material, over runs
+ * of planes of 56 x 14 nodes; the fields are the same bits on all of them. Any value
  * 0 keeps the current one. TETM_E_ARG for other values. */
 int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chunk_z);
 

@@ -311,17 +311,65 @@ void tetm::dev_free(void* p, cudaStream_t st) {
   if (p) cudaFreeAsync(p, st);
 }
 
-// The items (tile, chunk of cz planes) that own a field-carrying cell, in grid
-// order: items that run at the same time are neighbours and share their halo
-// rows through L2 (ordering the list by work instead was measured 1.3x slower).
-void tetm::work_list(const tetm_solver* s, int cz, std::vector<int>* list) {
-  const int nz = s->L.nz, tiles = s->tiles_x * s->tiles_y;
+namespace {
+
+// per tile of tx x ty nodes and plane (tile-major): 1 where one of its own
+// cells carries a field
+int tile_planes(tetm_solver* s, int tx, int ty, std::vector<uint8_t>* act) {
+  const Layout& L = s->L;
+  const int tiles_x = (L.nx + tx - 1) / tx, tiles_y = (L.ny + ty - 1) / ty;
+  const size_t n = (size_t)tiles_x * tiles_y * L.nz;
+  uint8_t* d = nullptr;
+  CK(dev_alloc((void**)&d, n, s->stream));
+  tile_activity<<<(unsigned)std::min<size_t>((n + 7) / 8, 1u << 16), 256, 0, s->stream>>>(
+      s->mask, L, tx, ty, tiles_x, (long long)n, d);
+  act->resize(n);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(act->data(), d, n, cudaMemcpyDeviceToHost, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  dev_free(d, s->stream);
+  return e == cudaSuccess ? TETM_OK : cuda_fail(e);
+}
+
+// The items (tile, chunk of cz planes) with an active plane, in grid order:
+// items that run at the same time are neighbours and share their halo rows
+// through L2 (ordering the list by work instead was measured 1.3x slower).
+void items_of(const std::vector<uint8_t>& act, int nz, int cz, std::vector<int>* list) {
+  const int tiles = (int)(act.size() / (size_t)nz);
   list->clear();
   for (int k0 = 0, c = 0; k0 < nz; k0 += cz, ++c)
     for (int t = 0; t < tiles; ++t)
-      if (memchr(s->act.data() + (size_t)t * nz + k0, 1, (size_t)std::min(cz, nz - k0)))
-        list->push_back(c * tiles + t);
+      if (memchr(act.data() + (size_t)t * nz + k0, 1, (size_t)std::min(cz, nz - k0))) list->push_back(c * tiles + t);
 }
+
+// items[cz]: how many those are, cz = lo .. hi
+std::vector<long long> count_items(const std::vector<uint8_t>& act, int nz, int lo, int hi) {
+  std::vector<long long> items((size_t)hi + 1, 0);
+  std::vector<int> before((size_t)nz + 1);  // active planes of the tile below a plane
+  for (size_t t = 0; t < act.size() / (size_t)nz; ++t) {
+    before[0] = 0;
+    for (int k = 0; k < nz; ++k) before[(size_t)k + 1] = before[(size_t)k] + act[t * nz + k];
+    if (!before[(size_t)nz]) continue;
+    for (int cz = lo; cz <= hi; ++cz)
+      for (int k0 = 0; k0 < nz; k0 += cz)
+        items[(size_t)cz] += before[(size_t)std::min(k0 + cz, nz)] > before[(size_t)k0];
+  }
+  return items;
+}
+
+int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return sms;
+}
+
+}  // namespace
+
+void tetm::work_list(const tetm_solver* s, int cz, std::vector<int>* list) { items_of(s->act, s->L.nz, cz, list); }
 
 // Planes per work item of the slab kernel, where the caller set none. Every
 // item takes about cz + 2 planes' time (the plane below the chunk, and filling
@@ -336,27 +384,12 @@ void tetm::work_list(const tetm_solver* s, int cz, std::vector<int>* list) {
 // the last one counts by half: items * share / slots + 1/2 on average, at least
 // one, and no more than kChunk planes, since the others may leave early (a batch
 // of 16: 406 ms at 20 to 32 planes, 441 at 8, 423 at 64).
-int tetm::choose_chunk(const tetm_solver* s, int share) {
-  const int nz = s->L.nz, tiles = s->tiles_x * s->tiles_y;
+int tetm::choose_chunk(const tetm_solver* s, int share, double* out) {
+  const int nz = s->L.nz, sms = sm_count();
   const int top = std::min(share == 1 ? kMaxChunk : kChunk, std::max(nz, kMinChunk));
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-    cudaGetLastError();
-    return kChunk;
-  }
+  if (sms < 1) return kChunk;
   const double slots = 2.0 * sms;
-  std::vector<long long> items((size_t)top + 1, 0);
-  std::vector<int> before((size_t)nz + 1);  // active planes of the tile below a plane
-  for (int t = 0; t < tiles; ++t) {
-    const uint8_t* a = s->act.data() + (size_t)t * nz;
-    before[0] = 0;
-    for (int k = 0; k < nz; ++k) before[(size_t)k + 1] = before[(size_t)k] + a[k];
-    if (!before[(size_t)nz]) continue;
-    for (int cz = kMinChunk; cz <= top; ++cz)
-      for (int k0 = 0; k0 < nz; k0 += cz)
-        items[(size_t)cz] += before[(size_t)std::min(k0 + cz, nz)] > before[(size_t)k0];
-  }
+  const std::vector<long long> items = count_items(s->act, nz, kMinChunk, top);
   int best = kMinChunk;
   double least = 0.0;
   for (int cz = kMinChunk; cz <= top; ++cz) {
@@ -367,6 +400,7 @@ int tetm::choose_chunk(const tetm_solver* s, int share) {
       least = cost;
     }
   }
+  if (out) *out = least;
   return best;
 }
 
@@ -382,17 +416,8 @@ int tetm::rebuild_work(tetm_solver* s) {
     dev_free(s->work, s->stream);
     s->work = nullptr;
   }
-  const size_t n = (size_t)tiles * L.nz;
-  uint8_t* act = nullptr;
-  CK(dev_alloc((void**)&act, n, s->stream));
-  tile_activity<<<(unsigned)std::min<size_t>((n + 7) / 8, 1u << 16), 256, 0, s->stream>>>(
-      s->mask, L, s->tile_x, rows, s->tiles_x, (long long)n, act);
-  s->act.resize(n);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s->act.data(), act, n, cudaMemcpyDeviceToHost, s->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  dev_free(act, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e);
+  const int rc = tile_planes(s, s->tile_x, rows, &s->act);
+  if (rc != TETM_OK) return rc;
   if (!s->own_chunk) s->chunk_z = s->auto_chunk() ? choose_chunk(s, 1) : kChunk;
   s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
   std::vector<int> list;
@@ -439,6 +464,42 @@ int build_band(tetm_solver* s) {
   const int rc = dalloc(s, (void**)&s->band, sizeof(int4) * items.size());
   if (rc != TETM_OK) return rc;
   CK(cudaMemcpyAsync(s->band, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s->stream));
+  CK(cudaStreamSynchronize(s->stream));
+  return TETM_OK;
+}
+
+// Work items of the half-step kernels, where they are the faster float32 step
+// (none otherwise). An item of `run` planes takes about run + 2 planes' time
+// (its two launches each fill once), kHalfBlocks of them per SM at once, in the
+// units of choose_chunk as long as latency bounds both. Up to kHalfCells active
+// cells it does: us per step on the sweep | the halves at the run chosen here,
+// 10.2 | 4.1 at 7e3 active cells, 10.2 | 5.2 at 1.1e5, 12.3 | 7.9 at 2.9e5,
+// 14.4 | 10.8 at 3.7e5, 20.5 | 14.7 at 6.3e5; beyond, the halves' fuller SMs and
+// 64 bytes per node cost more: 20.5 | 21.2 at 8.7e5, 28.7 | 31.8 at 1.4e6.
+constexpr long long kHalfCells = 3LL << 18;
+int build_half(tetm_solver* s) {
+  const int nz = s->L.nz, sms = sm_count();
+  if (sms < 1 || s->n_work == 0 || s->active_cells > kHalfCells) return TETM_OK;
+  double sweep = 0.0;
+  choose_chunk(s, 1, &sweep);
+  const double slots = (double)kHalfBlocks * sms;
+  std::vector<uint8_t> act;
+  int rc = tile_planes(s, kHalfX, kHalfY, &act);
+  if (rc != TETM_OK) return rc;
+  const std::vector<long long> items = count_items(act, nz, 1, kMaxRun);
+  for (int run = 1; run <= kMaxRun; ++run) {
+    const double cost = ceil((double)items[(size_t)run] / slots) * (run + 2);
+    if (cost >= sweep) continue;
+    s->half_run = run;
+    sweep = cost;
+  }
+  if (!s->half_run) return TETM_OK;
+  std::vector<int> list;
+  items_of(act, nz, s->half_run, &list);
+  s->n_half = (int)list.size();
+  rc = dalloc(s, (void**)&s->half, sizeof(int) * list.size());
+  if (rc != TETM_OK) return rc;
+  CK(cudaMemcpyAsync(s->half, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   return TETM_OK;
 }
@@ -595,10 +656,14 @@ int do_steps(tetm_solver* s, int n) {
     } else if (s->kernel == TETM_KERNEL_FUSED) {
       StepArgs<T> a = step_args<T>(s, true);
       if (s->n_work > 0) {
-        bool band = false;
+        bool band = false, half = false;
         if constexpr (sizeof(T) == 8) band = s->band && !s->own_shape;
+        if constexpr (sizeof(T) == 4) half = s->half && !s->own_shape;
         if (band) {
           if constexpr (sizeof(T) == 8) CK(launch_band_step(a, s->band, s->n_band, s->band_smem, s->stream));
+        } else if (half) {  // with the transverse wake
+          if constexpr (sizeof(T) == 4) CK(launch_half_step(a, s->half, s->n_half, s->half_run, s->stream));
+          a.b.obs_on = 0;
         } else if (warp_shape_ok(s->tile_x, s->tile_y)) {
           CK(launch_fused_warp_step<T>(a, s->tile_x, s->tile_y, s->stream));
         } else if (slab_shape_ok(s->tile_x, s->tile_y, !s->uniform)) {
@@ -611,7 +676,7 @@ int do_steps(tetm_solver* s, int n) {
           CK(launch_fused_step<T>(a, s->tile_x, s->tile_y, s->stream));
         }
       }
-      if (s->bunch && s->obs_on) CK(launch_transverse_after_step<T>(a, s->stream));
+      if (a.b.obs_on) CK(launch_transverse_after_step<T>(a, s->stream));
       s->cur = 1 - s->cur;
     } else {
       if (q == n - 1 || bal) {  // keep y^n beside y^{n+1} for the charge balance
@@ -691,6 +756,7 @@ void free_all(tetm_solver* s) {
   dev_free(s->mask, st);
   dev_free(s->work, st);
   dev_free(s->band, st);
+  dev_free(s->half, st);
   dev_free(s->J, st);
   dev_free(s->W, st);
   dev_free(s->qline, st);
@@ -899,6 +965,7 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   if (rc == TETM_OK) rc = rebuild_work(s);
   // (a z-slab keeps the fused sweep, which recomputes its ghost plane's TM half)
   if (rc == TETM_OK && s->esz == 8 && !s->is_slab()) rc = build_band(s);
+  if (rc == TETM_OK && s->esz == 4 && s->uniform && !s->is_slab()) rc = build_half(s);
   if (rc != TETM_OK) {
     free_all(s);
     delete s;

@@ -72,18 +72,19 @@ __device__ __forceinline__ void add_wake(const BunchDev<T>& b, long long m, T ez
 
 // Transverse wake samples of plane k (step n -> n+1): W_x from the old e_x
 // and the new h_y of the x-edge at the observer line, W_y from the old e_y
-// and the new h_x of the y-edge; sample m = n + kshift - k - c0 as for W.
+// and the new h_x of the y-edge; sample m = n + kshift - k - c0 as for W, one
+// addition as there.
 template <typename T>
 __device__ __forceinline__ void gather_wx(const BunchDev<T>& b, long long n, int k, T ex_old, T hy_new) {
   const long long mm = (n + b.kshift) - k - b.c0;
   if (mm >= b.m_min && mm <= b.m_max)
-    b.WX[mm - b.m_min] += b.tw_ex * (double)ex_old + b.tw_hy * (double)hy_new;
+    atomicAdd(b.WX + (mm - b.m_min), b.tw_ex * (double)ex_old + b.tw_hy * (double)hy_new);
 }
 template <typename T>
 __device__ __forceinline__ void gather_wy(const BunchDev<T>& b, long long n, int k, T ey_old, T hx_new) {
   const long long mm = (n + b.kshift) - k - b.c0;
   if (mm >= b.m_min && mm <= b.m_max)
-    b.WY[mm - b.m_min] += b.tw_ey * (double)ey_old + b.tw_hx * (double)hx_new;
+    atomicAdd(b.WY + (mm - b.m_min), b.tw_ey * (double)ey_old + b.tw_hx * (double)hx_new);
 }
 
 // Per-component coefficients: either one constant per component with the
@@ -165,6 +166,12 @@ cudaError_t launch_fused_slab_batch(BatchMember<float>* members, int n_members, 
 // kernel's dynamic schedule uses and leaves zero (nullptr: static order)
 // (a.co.ua[0] set: the per-entry coefficient arrays of material runs)
 cudaError_t launch_fused_slab_step(const StepArgs<float>& a, int* sched, cudaStream_t st);
+
+// ---- float32 step of a small grid in two launches (kernels_half.cu), with the
+// transverse wake: items of kHalfX x kHalfY nodes of `run` planes, numbered
+// tile + tiles * run index, kHalfBlocks resident per SM -----------------------
+constexpr int kHalfX = 56, kHalfY = 14, kHalfBlocks = 4, kMaxRun = 8;
+cudaError_t launch_half_step(const StepArgs<float>& a, const int* items, int n, int run, cudaStream_t st);
 
 // ---- float64 step in two launches over bands of planes (kernels_band.cu) ---
 // the work items: int4 {plane, first row, first column, columns | rows << 16},
@@ -283,6 +290,8 @@ struct tetm_solver {
   std::vector<uint8_t> act;    // per tile and plane (tile-major): the tile owns an active cell there
   int4* band;                  // float64: work items of the band kernels (the default work shape)
   int n_band, band_smem;
+  int* half;                   // float32, small grids: work items of the half-step kernels (tile + tiles * run)
+  int n_half, half_run;        // planes per item
   std::vector<int> work_host;  // host copy of the work list
   // the slab kernel's shape: planes per item by choose_chunk unless set
   bool auto_chunk() const { return esz == 4 && tetm::slab_shape_ok(tile_x, tile_y, !uniform); }
@@ -350,7 +359,7 @@ int rebuild_work(tetm_solver* s);
 constexpr int kChunk = 32, kMinChunk = 4, kMaxChunk = 64;  // planes per work item: set ones start at kMinChunk
 // the slab kernel's planes per item for one of `share` solves that step
 // together, and the items of chunks of cz planes (both from s->act)
-int choose_chunk(const tetm_solver* s, int share);
+int choose_chunk(const tetm_solver* s, int share, double* cost = nullptr);
 void work_list(const tetm_solver* s, int cz, std::vector<int>* list);
 // Device memory of solves and batches comes from one stream-ordered pool per
 // device: allocation and release are queued on the given stream, so neither
