@@ -113,53 +113,79 @@ struct MinvOut {
   double* a[6];  // per-entry M^-1 arrays (material runs) or nullptr
 };
 
-// Activity bits (and M^-1 arrays) of the node entries of planes k_first ..
-// nz: k_first = 0 for a whole grid, -1 for a z-slab whose plane below its
-// first one is a ghost plane with the geometry of the whole grid.
-__global__ void build_geometry(GeomIn g, Layout L, int k_first, uint8_t* mask, MinvOut mo) {
-  const long long total = (long long)(g.nx + 1) * (g.ny + 1) * (g.nz + 1 - k_first);
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= total) return;
-  const int i = (int)(q % (g.nx + 1));
-  const int j = (int)((q / (g.nx + 1)) % (g.ny + 1));
-  const int k = k_first + (int)(q / ((long long)(g.nx + 1) * (g.ny + 1)));
-  const long long id = L.idx(i, j, k);
-  double v[6] = {0, 0, 0, 0, 0, 0};
-  const bool kin = k + g.k_off < g.nz_all;  // the edge or face along z lies inside the whole grid
-  if (i < g.nx) v[kEX] = edge_minv(g, 0, i, j, k);
-  if (j < g.ny) v[kEY] = edge_minv(g, 1, i, j, k);
-  if (kin) v[kEZ] = edge_minv(g, 2, i, j, k);
-  if (j < g.ny && kin) v[kHX] = face_minv(g, 0, i, j, k);
-  if (i < g.nx && kin) v[kHY] = face_minv(g, 1, i, j, k);
-  if (i < g.nx && j < g.ny) v[kHZ] = face_minv(g, 2, i, j, k);
-  uint8_t m = 0;
-  for (int c = 0; c < 6; ++c) {
-    if (v[c] != 0.0) m |= (uint8_t)(1u << c);
-    if (mo.a[c]) mo.a[c][id] = v[c];
+// Activity bits (and M^-1 arrays, zero on entry) of the node entries of planes
+// k_first .. nz: k_first = 0 for a whole grid, -1 for a z-slab whose plane
+// below its first one is a ghost plane with the geometry of the whole grid; the
+// nodes 0 .. n-1 of planes 0 .. nz-1 that carry a field are added to *active.
+// Every entry of a node touches the node's own cell, so a node of a PEC cell
+// has none, and with one material (no arrays) an entry carries a field where
+// the cells around it are open and its constant is not zero (a bit of live).
+// The six float64 quotients per node, which the mask alone does not need, were
+// the time: 4.9 ms for 256 x 256 x 1024 nodes, so 0.3; with arrays the PEC part
+// is spared, 2.7 -> 1.5 ms for 192 x 192 x 768 nodes with a quarter open. (The
+// activity count, a pass of its own, took 0.7 ms on the former.)
+template <bool ARRAYS>
+__global__ void __launch_bounds__(256) build_geometry(GeomIn g, Layout L, int k_first, unsigned per_plane, unsigned live,
+                                                      uint8_t* mask, MinvOut mo, unsigned long long* active) {
+  const int k = k_first + (int)(blockIdx.x / per_plane);
+  const unsigned q = (blockIdx.x % per_plane) * blockDim.x + threadIdx.x;
+  const int i = (int)(q % (unsigned)(g.nx + 1)), j = (int)(q / (unsigned)(g.nx + 1));
+  unsigned m = 0;
+  if (j <= g.ny && !gpec(g, i, j, k)) {
+    const long long id = L.idx(i, j, k);
+    if constexpr (ARRAYS) {
+      const double v[6] = {edge_minv(g, 0, i, j, k), edge_minv(g, 1, i, j, k), edge_minv(g, 2, i, j, k),
+                           face_minv(g, 0, i, j, k), face_minv(g, 1, i, j, k), face_minv(g, 2, i, j, k)};
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        if (v[c] != 0.0) m |= 1u << c;
+        mo.a[c][id] = v[c];
+      }
+    } else {
+      const bool x = !gpec(g, i - 1, j, k), y = !gpec(g, i, j - 1, k), z = !gpec(g, i, j, k - 1);
+      if (y && z && !gpec(g, i, j - 1, k - 1)) m |= 1u << kEX;
+      if (x && z && !gpec(g, i - 1, j, k - 1)) m |= 1u << kEY;
+      if (x && y && !gpec(g, i - 1, j - 1, k)) m |= 1u << kEZ;
+      if (x) m |= 1u << kHX;
+      if (y) m |= 1u << kHY;
+      if (z) m |= 1u << kHZ;
+      m &= live;
+    }
+    mask[id] = (uint8_t)m;
   }
-  mask[id] = m;
+  const int n = __syncthreads_count(m != 0 && k >= 0 && k < g.nz);  // (the cell (i, j, k) is open: i < nx, j < ny)
+  if (threadIdx.x == 0 && n) atomicAdd(active, (unsigned long long)n);
 }
 
+// The update coefficients of one component from its M^-1: s M^-1 for the
+// steps and, for the balances, which would otherwise divide at every use, M =
+// 1 / M^-1 in float64 (m) or as a (hi, lo) float32 pair whose sum is the float64
+// value to 2^-48 (mp), and a2 M^-1 as a pair (ap), each where its array is
+// given; 0 where M^-1 is 0 (an entry without a field, in most warps a whole one,
+// which skips the float64 arithmetic). One pass; a kernel per array over all
+// entries took 6.2 ms for 192 x 192 x 768 nodes in float32.
 template <typename T>
-__global__ void scale_coef(const double* minv, double s, long long n, T* out) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n) out[q] = (T)(s * minv[q]);
-}
-// M = 1/M^-1 per entry (0 where M^-1 is 0: an entry without a field), for the
-// balances, which would otherwise divide at every use
-__global__ void recip_coef(const double* minv, long long n, double* out) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n) out[q] = minv[q] != 0.0 ? 1.0 / minv[q] : 0.0;
-}
-// The same (recip) or s M^-1 as a (hi, lo) float32 pair whose sum is the
-// float64 value to 2^-48, for the float32-pair balances
-__global__ void pair_coef(const double* minv, double s, bool recip, long long n, float2* out) {
+__global__ void entry_coefs(const double* minv, double s, double a2, long long n, T* u, double* m, float2* mp, float2* ap) {
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n) return;
   const double v = minv[q];
-  const double x = recip ? (v != 0.0 ? 1.0 / v : 0.0) : s * v;
-  const float hi = (float)x;
-  out[q] = make_float2(hi, (float)(x - (double)hi));
+  auto pair = [](double x) {
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
+  };
+  T uq = 0;
+  double r = 0.0;
+  float2 p = make_float2(0.f, 0.f), a = p;
+  if (v != 0.0) {
+    uq = (T)(s * v);
+    r = 1.0 / v;
+    if (mp) p = pair(r);
+    if (ap) a = pair(a2 * v);
+  }
+  u[q] = uq;
+  if (m) m[q] = r;
+  if (mp) mp[q] = p;
+  if (ap) ap[q] = a;
 }
 
 // Canonical FIT layout <-> device layout, for planes [k0, k0 + nk).
@@ -216,18 +242,6 @@ __global__ void guard_scan(const T* f, const uint8_t* mask, long long count, int
     if (f[q] != T(0) && !((mask[q] >> comp) & 1)) ++c;
   for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
-}
-
-__global__ void count_active(const uint8_t* mask, Layout L, unsigned long long* out) {
-  const long long total = (long long)L.nx * L.ny * L.nz;
-  unsigned long long c = 0;
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(q % L.nx), j = (int)((q / L.nx) % L.ny), k = (int)(q / ((long long)L.nx * L.ny));
-    c += mask[L.idx(i, j, k)] != 0;
-  }
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out, c);
 }
 
 double phi(double x) { return 0.5 * erfc(-x / sqrt(2.0)); }
@@ -903,12 +917,33 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
     gi.eps = deps;
     gi.mu = dmu;
   }
+  unsigned long long* cnt = nullptr;
+  if (rc == TETM_OK && dev_alloc((void**)&cnt, sizeof(*cnt), s->stream) != cudaSuccess) rc = TETM_E_CUDA;
   if (rc == TETM_OK) {
     const int k_first = k_lo > 0 ? -1 : 0;  // a z-slab's ghost plane below takes the whole grid's geometry
-    const long long total = (long long)(g->nx + 1) * (g->ny + 1) * (g->nz + 1 - k_first);
-    build_geometry<<<(unsigned)((total + 255) / 256), 256, 0, s->stream>>>(gi, s->L, k_first, s->mask, mo);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s->stream) != cudaSuccess) rc = TETM_E_CUDA;
+    const unsigned per_plane = (unsigned)(((long long)(g->nx + 1) * (g->ny + 1) + 255) / 256);
+    const long long blocks = (long long)per_plane * (g->nz + 1 - k_first);
+    // the components whose M^-1 is not zero with one material
+    const double e = kEps0 * 0.25 * 4.0, h = 0.5 * 2.0;
+    const double v[6] = {g->dx / (e * (g->dy * g->dz)), g->dy / (e * (g->dx * g->dz)), g->dz / (e * (g->dx * g->dy)),
+                         g->dx * h / (kMu0 * (g->dy * g->dz)), g->dy * h / (kMu0 * (g->dx * g->dz)),
+                         g->dz * h / (kMu0 * (g->dx * g->dy))};
+    unsigned live = 0;
+    for (int c = 0; c < 6; ++c)
+      if (v[c] != 0.0) live |= 1u << c;
+    unsigned long long n = 0;
+    cudaMemsetAsync(cnt, 0, sizeof(*cnt), s->stream);
+    if (mo.a[0])
+      build_geometry<true><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, mo, cnt);
+    else
+      build_geometry<false><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, mo, cnt);
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemcpyAsync(&n, cnt, sizeof(n), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
+        cudaStreamSynchronize(s->stream) != cudaSuccess)
+      rc = TETM_E_CUDA;
+    s->active_cells = (long long)n;
   }
+  dev_free(cnt, s->stream);
   dev_free(dpec, s->stream);
   dev_free(deps, s->stream);
   dev_free(dmu, s->stream);
@@ -933,34 +968,18 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
         const bool a2 = c == kHX || c == kHY || c == kEX || c == kEY;
         rc = dalloc(s, (void**)&s->mp[c], sizeof(float2) * (size_t)s->L.count);
         if (rc == TETM_OK && a2) rc = dalloc(s, (void**)&s->ap[c], sizeof(float2) * (size_t)s->L.count);
-        if (rc != TETM_OK) break;
-        pair_coef<<<nb, 256, 0, s->stream>>>(s->minv_a[c], 0.0, true, s->L.count, s->mp[c]);
-        if (a2) pair_coef<<<nb, 256, 0, s->stream>>>(s->minv_a[c], s->alpha * s->alpha, false, s->L.count, s->ap[c]);
       } else {
         rc = dalloc(s, (void**)&s->m_a[c], sizeof(double) * (size_t)s->L.count);
-        if (rc != TETM_OK) break;
-        recip_coef<<<nb, 256, 0, s->stream>>>(s->minv_a[c], s->L.count, s->m_a[c]);
       }
+      if (rc != TETM_OK) break;
       if (s->esz == 8)
-        scale_coef<double><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, s->L.count, (double*)s->ua[c]);
+        entry_coefs<double><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, 0.0, s->L.count, (double*)s->ua[c], s->m_a[c],
+                                                       nullptr, nullptr);
       else
-        scale_coef<float><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, s->L.count, (float*)s->ua[c]);
+        entry_coefs<float><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, s->alpha * s->alpha, s->L.count,
+                                                      (float*)s->ua[c], nullptr, s->mp[c], s->ap[c]);
       if (cudaGetLastError() != cudaSuccess) rc = TETM_E_CUDA;
     }
-  }
-  if (rc == TETM_OK) {
-    unsigned long long* cnt = nullptr;
-    unsigned long long h = 0;
-    if (dev_alloc((void**)&cnt, sizeof(*cnt), s->stream) != cudaSuccess) rc = TETM_E_CUDA;
-    if (rc == TETM_OK) {
-      cudaMemsetAsync(cnt, 0, sizeof(*cnt), s->stream);
-      count_active<<<256, 256, 0, s->stream>>>(s->mask, s->L, cnt);
-      if (cudaMemcpyAsync(&h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
-          cudaStreamSynchronize(s->stream) != cudaSuccess)
-        rc = TETM_E_CUDA;
-      dev_free(cnt, s->stream);
-    }
-    s->active_cells = (long long)h;
   }
   if (rc == TETM_OK) rc = rebuild_work(s);
   // (a z-slab keeps the fused sweep, which recomputes its ghost plane's TM half)
