@@ -157,6 +157,19 @@ __global__ void __launch_bounds__(256) build_geometry(GeomIn g, Layout L, int k_
   if (threadIdx.x == 0 && n) atomicAdd(active, (unsigned long long)n);
 }
 
+// flags |= 1: a value is not a finite number >= 1, |= 2: not all are equal
+__global__ void scan_cells(const double* a, long long n, int* flags) {
+  const double first = a[0];
+  int f = 0;
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
+    const double v = a[q];
+    if (!(v >= 1.0) || !isfinite(v)) f |= 1;
+    if (v != first) f |= 2;
+  }
+  f = __reduce_or_sync(0xffffffffu, f);
+  if ((threadIdx.x & 31) == 0 && f) atomicOr(flags, f);
+}
+
 // The update coefficients of one component from its M^-1: s M^-1 for the
 // steps and, for the balances, which would otherwise divide at every use, M =
 // 1 / M^-1 in float64 (m) or as a (hi, lo) float32 pair whose sum is the float64
@@ -813,6 +826,61 @@ int64_t tetm_bytes_needed(const tetm_grid* g) {
 
 namespace {
 
+// The flags of scan_cells for an array of n host values, which stays on the
+// device in *out; -1 with nothing there where the device cannot.
+int scan_on_device(const double* a, long long n, cudaStream_t st, double** out) {
+  double* d = nullptr;
+  int *f = nullptr, h = -1;
+  if (dev_alloc((void**)&d, sizeof(double) * (size_t)n, st) == cudaSuccess &&
+      dev_alloc((void**)&f, sizeof(int), st) == cudaSuccess && cudaMemsetAsync(f, 0, sizeof(int), st) == cudaSuccess &&
+      cudaMemcpyAsync(d, a, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice, st) == cudaSuccess) {
+    scan_cells<<<1024, 256, 0, st>>>(d, n, f);
+    if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(&h, f, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      h = -1;
+  }
+  dev_free(f, st);
+  if (h < 0) {
+    dev_free(d, st);
+    d = nullptr;
+    cudaGetLastError();
+  }
+  *out = d;
+  return h;
+}
+
+// Checks the material arrays (every value a finite number >= 1) and whether
+// each holds one value only. On the host a pass over an array takes 0.74 ns per
+// cell (20.9 ms for the 2.8e7 cells of a 192 x 192 x 768 grid), on the device
+// its upload, which the geometry of a grid with several materials needs anyway,
+// and 0.05 ms; so above kScanCells the arrays go up first and stay in dcell when
+// they are not uniform. Where the device refuses (none there, no memory left)
+// the host looks, so that a wrong value is a wrong argument there too.
+constexpr long long kScanCells = 1 << 16;  // 48 us on the host, as much as a launch and its two copies
+int cell_materials(const double* eps_r, const double* mu_r, long long ncell, cudaStream_t st, bool* uniform,
+                   double* dcell[2]) {
+  int flags = 0;
+  for (int w = 0; w < 2; ++w) {
+    const double* a = w == 0 ? eps_r : mu_r;
+    if (!a) continue;
+    int f = -1;
+    if (ncell > kScanCells) f = scan_on_device(a, ncell, st, &dcell[w]);
+    if (f < 0) {
+      f = 0;
+      for (long long q = 0; q < ncell && !(f & 1); ++q) f |= (!(a[q] >= 1.0) || !isfinite(a[q]) ? 1 : 0) | (a[q] != a[0] ? 2 : 0);
+    }
+    flags |= f;
+    if (f & 1) break;
+  }
+  *uniform = !(flags & 2);
+  if (*uniform || (flags & 1))
+    for (int w = 0; w < 2; ++w) {
+      dev_free(dcell[w], st);
+      dcell[w] = nullptr;
+    }
+  return flags & 1 ? TETM_E_ARG : TETM_OK;
+}
+
 // A solve of planes [k_lo, k_lo + g->nz) of a grid of nz_all planes (the
 // whole grid: k_lo = 0, nz_all = g->nz); the cell arrays cover the whole grid.
 int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, const double* mu_r,
@@ -827,22 +895,21 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   // materials: physical (>= 1) and finite; uniform if every cell has the same value
   bool uniform = true;
   double eps_u = 1.0, mu_u = 1.0;
-  for (int w = 0; w < 2; ++w) {
-    const double* a = w == 0 ? eps_r : mu_r;
-    if (!a) continue;
-    for (long long q = 0; q < ncell; ++q)
-      if (!(a[q] >= 1.0) || !isfinite(a[q])) return TETM_E_ARG;
-    for (long long q = 1; q < ncell; ++q)
-      if (a[q] != a[0]) { uniform = false; break; }
-    (w == 0 ? eps_u : mu_u) = a[0];
-  }
+  double* dcell[2] = {nullptr, nullptr};  // eps_r, mu_r on the device (not uniform)
+  const int checked = cell_materials(eps_r, mu_r, ncell, st, &uniform, dcell);
+  if (checked != TETM_OK) return checked;
+  if (eps_r) eps_u = eps_r[0];
+  if (mu_r) mu_u = mu_r[0];
   int dev_count = 0;
   if (cudaGetDeviceCount(&dev_count) != cudaSuccess || dev_count < 1) {
     cudaGetLastError();
     return TETM_E_CUDA;
   }
   tetm_solver* s = new (std::nothrow) tetm_solver();
-  if (!s) return TETM_E_NOMEM;
+  if (!s) {
+    for (double* d : dcell) dev_free(d, st);
+    return TETM_E_NOMEM;
+  }
   s->g = *g;
   s->g.cdt = cdt;
   s->k_lo = k_lo;
@@ -898,7 +965,6 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   gi.nz_all = nz_all;
   gi.dx = g->dx; gi.dy = g->dy; gi.dz = g->dz;
   uint8_t* dpec = nullptr;
-  double *deps = nullptr, *dmu = nullptr;
   if (rc == TETM_OK && pec) {
     if (dev_alloc((void**)&dpec, (size_t)ncell, s->stream) != cudaSuccess ||
         cudaMemcpyAsync(dpec, pec, (size_t)ncell, cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
@@ -908,14 +974,13 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   if (rc == TETM_OK && !uniform) {
     for (int w = 0; w < 2 && rc == TETM_OK; ++w) {
       const double* a = w == 0 ? eps_r : mu_r;
-      if (!a) continue;
-      double** d = w == 0 ? &deps : &dmu;
-      if (dev_alloc((void**)d, sizeof(double) * (size_t)ncell, s->stream) != cudaSuccess ||
-          cudaMemcpyAsync(*d, a, sizeof(double) * (size_t)ncell, cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
+      if (a && !dcell[w] &&
+          (dev_alloc((void**)&dcell[w], sizeof(double) * (size_t)ncell, s->stream) != cudaSuccess ||
+           cudaMemcpyAsync(dcell[w], a, sizeof(double) * (size_t)ncell, cudaMemcpyHostToDevice, s->stream) != cudaSuccess))
         rc = TETM_E_CUDA;
     }
-    gi.eps = deps;
-    gi.mu = dmu;
+    gi.eps = dcell[0];
+    gi.mu = dcell[1];
   }
   unsigned long long* cnt = nullptr;
   if (rc == TETM_OK && dev_alloc((void**)&cnt, sizeof(*cnt), s->stream) != cudaSuccess) rc = TETM_E_CUDA;
@@ -945,8 +1010,7 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   }
   dev_free(cnt, s->stream);
   dev_free(dpec, s->stream);
-  dev_free(deps, s->stream);
-  dev_free(dmu, s->stream);
+  for (double* d : dcell) dev_free(d, s->stream);
   // per-component constants for the uniform case (vacuum or one material)
   const double dx = g->dx, dy = g->dy, dz = g->dz;
   s->minv_c[kEX] = dx / (kEps0 * eps_u * dy * dz);
