@@ -109,11 +109,38 @@ __device__ double face_minv(const GeomIn& g, int axis, long i, long j, long k) {
   return len * 0.5 * r / (kMu0 * area);
 }
 
-struct MinvOut {
-  double* a[6];  // per-entry M^-1 arrays (material runs) or nullptr
+// Per-entry arrays of a component (material runs; nullptr where not kept): the
+// steps' coefficient s M^-1 and, for the balances, which would otherwise divide
+// at every use, M^-1 and M in float64 (float64 fields) or M and a2 M^-1 as
+// (hi, lo) float32 pairs whose sum is the float64 value to 2^-48 (float32).
+struct EntryOut {
+  void* u;
+  double s;
+  double *minv, *m;
+  float2 *mp, *ap;
+  double a2;
 };
+struct EntryOuts {
+  EntryOut c[6];
+};
+template <typename T>
+__device__ __forceinline__ void put_entry(const EntryOut& o, long long id, double v) {
+  auto pair = [](double x) {
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
+  };
+  if (v == 0.0) return;
+  static_cast<T*>(o.u)[id] = (T)(o.s * v);
+  if constexpr (sizeof(T) == 8) {
+    o.minv[id] = v;
+    o.m[id] = 1.0 / v;
+  } else {
+    o.mp[id] = pair(1.0 / v);
+    if (o.ap) o.ap[id] = pair(o.a2 * v);
+  }
+}
 
-// Activity bits (and M^-1 arrays, zero on entry) of the node entries of planes
+// Activity bits (and the per-entry arrays, zero on entry) of the node entries of planes
 // k_first .. nz: k_first = 0 for a whole grid, -1 for a z-slab whose plane
 // below its first one is a ghost plane with the geometry of the whole grid; the
 // nodes 0 .. n-1 of planes 0 .. nz-1 that carry a field are added to *active.
@@ -121,12 +148,14 @@ struct MinvOut {
 // has none, and with one material (no arrays) an entry carries a field where
 // the cells around it are open and its constant is not zero (a bit of live).
 // The six float64 quotients per node, which the mask alone does not need, were
-// the time: 4.9 ms for 256 x 256 x 1024 nodes, so 0.3; with arrays the PEC part
-// is spared, 2.7 -> 1.5 ms for 192 x 192 x 768 nodes with a quarter open. (The
-// activity count, a pass of its own, took 0.7 ms on the former.)
-template <bool ARRAYS>
+// the time: 4.9 ms for 256 x 256 x 1024 nodes, so 0.3 (and the activity count, a
+// pass of its own, 0.7). With arrays the entries' M^-1 become their
+// coefficients here and only float64 fields keep them: in arrays of their own
+// they were a quarter of the device memory of a float32 solve (1.5 GB for 192 x
+// 192 x 768 nodes), written, read back and released for 1.6 ms.
+template <typename T, bool ARRAYS>
 __global__ void __launch_bounds__(256) build_geometry(GeomIn g, Layout L, int k_first, unsigned per_plane, unsigned live,
-                                                      uint8_t* mask, MinvOut mo, unsigned long long* active) {
+                                                      uint8_t* mask, EntryOuts out, unsigned long long* active) {
   const int k = k_first + (int)(blockIdx.x / per_plane);
   const unsigned q = (blockIdx.x % per_plane) * blockDim.x + threadIdx.x;
   const int i = (int)(q % (unsigned)(g.nx + 1)), j = (int)(q / (unsigned)(g.nx + 1));
@@ -139,7 +168,7 @@ __global__ void __launch_bounds__(256) build_geometry(GeomIn g, Layout L, int k_
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         if (v[c] != 0.0) m |= 1u << c;
-        mo.a[c][id] = v[c];
+        put_entry<T>(out.c[c], id, v[c]);
       }
     } else {
       const bool x = !gpec(g, i - 1, j, k), y = !gpec(g, i, j - 1, k), z = !gpec(g, i, j, k - 1);
@@ -168,37 +197,6 @@ __global__ void scan_cells(const double* a, long long n, int* flags) {
   }
   f = __reduce_or_sync(0xffffffffu, f);
   if ((threadIdx.x & 31) == 0 && f) atomicOr(flags, f);
-}
-
-// The update coefficients of one component from its M^-1: s M^-1 for the
-// steps and, for the balances, which would otherwise divide at every use, M =
-// 1 / M^-1 in float64 (m) or as a (hi, lo) float32 pair whose sum is the float64
-// value to 2^-48 (mp), and a2 M^-1 as a pair (ap), each where its array is
-// given; 0 where M^-1 is 0 (an entry without a field, in most warps a whole one,
-// which skips the float64 arithmetic). One pass; a kernel per array over all
-// entries took 6.2 ms for 192 x 192 x 768 nodes in float32.
-template <typename T>
-__global__ void entry_coefs(const double* minv, double s, double a2, long long n, T* u, double* m, float2* mp, float2* ap) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  const double v = minv[q];
-  auto pair = [](double x) {
-    const float hi = (float)x;
-    return make_float2(hi, (float)(x - (double)hi));
-  };
-  T uq = 0;
-  double r = 0.0;
-  float2 p = make_float2(0.f, 0.f), a = p;
-  if (v != 0.0) {
-    uq = (T)(s * v);
-    r = 1.0 / v;
-    if (mp) p = pair(r);
-    if (ap) a = pair(a2 * v);
-  }
-  u[q] = uq;
-  if (m) m[q] = r;
-  if (mp) mp[q] = p;
-  if (ap) ap[q] = a;
 }
 
 // Canonical FIT layout <-> device layout, for planes [k0, k0 + nk).
@@ -946,16 +944,29 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   s->hist_cap = 4096;
   if (rc == TETM_OK) rc = dalloc(s, (void**)&s->hist, sizeof(double) * 5 * (size_t)s->hist_cap);
   if (rc == TETM_OK) rc = dalloc(s, (void**)&s->qline, sizeof(double) * (size_t)(g->nz + 1));
-  MinvOut mo;
-  for (int c = 0; c < 6; ++c) mo.a[c] = nullptr;
+  EntryOuts eo;
+  memset(&eo, 0, sizeof(eo));
   if (rc == TETM_OK && !uniform) {
-    for (int c = 0; c < 6 && rc == TETM_OK; ++c) {
-      rc = dalloc(s, (void**)&s->minv_a[c], sizeof(double) * (size_t)s->L.count);
-      if (rc == TETM_OK) rc = cudaMemsetAsync(s->minv_a[c], 0, sizeof(double) * (size_t)s->L.count, s->stream) == cudaSuccess ? TETM_OK : TETM_E_CUDA;
-      mo.a[c] = s->minv_a[c];
+    const size_t n = (size_t)s->L.count;
+    auto zeroed = [&](void** p, size_t bytes) {
+      if (rc == TETM_OK) rc = dalloc(s, p, bytes);
+      if (rc == TETM_OK && cudaMemsetAsync(*p, 0, bytes, s->stream) != cudaSuccess) rc = TETM_E_CUDA;
+    };
+    for (int c = 0; c < 6; ++c) {
+      const bool a2 = c == kHX || c == kHY || c == kEX || c == kEY;
+      zeroed(&s->ua[c], n * s->esz);
+      if (s->esz == 8) {
+        zeroed((void**)&s->minv_a[c], n * sizeof(double));
+        zeroed((void**)&s->m_a[c], n * sizeof(double));
+      } else {
+        zeroed((void**)&s->mp[c], n * sizeof(float2));
+        if (a2) zeroed((void**)&s->ap[c], n * sizeof(float2));
+      }
+      eo.c[c] = EntryOut{s->ua[c],    (c == kEZ || c == kHZ) ? 2.0 * s->alpha : s->alpha,
+                         s->minv_a[c], s->m_a[c], s->mp[c], s->ap[c], s->alpha * s->alpha};
     }
   }
-  // upload the cell arrays, build the mask (and M^-1 arrays) on the device
+  // upload the cell arrays, build the mask (and the per-entry arrays) on the device
   GeomIn gi;
   gi.pec = nullptr;
   gi.eps = nullptr;
@@ -998,10 +1009,12 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
       if (v[c] != 0.0) live |= 1u << c;
     unsigned long long n = 0;
     cudaMemsetAsync(cnt, 0, sizeof(*cnt), s->stream);
-    if (mo.a[0])
-      build_geometry<true><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, mo, cnt);
+    if (uniform)
+      build_geometry<float, false><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, eo, cnt);
+    else if (s->esz == 8)
+      build_geometry<double, true><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, eo, cnt);
     else
-      build_geometry<false><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, mo, cnt);
+      build_geometry<float, true><<<(unsigned)blocks, 256, 0, s->stream>>>(gi, s->L, k_first, per_plane, live, s->mask, eo, cnt);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(&n, cnt, sizeof(n), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
@@ -1019,32 +1032,6 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   s->minv_c[kHX] = dx / (kMu0 * mu_u * dy * dz);
   s->minv_c[kHY] = dy / (kMu0 * mu_u * dx * dz);
   s->minv_c[kHZ] = dz / (kMu0 * mu_u * dx * dy);
-  if (rc == TETM_OK && !uniform) {
-    for (int c = 0; c < 6 && rc == TETM_OK; ++c) {
-      rc = dalloc(s, &s->ua[c], (size_t)s->L.count * s->esz);
-      if (rc != TETM_OK) break;
-      const double sc = (c == kEZ || c == kHZ) ? 2.0 * s->alpha : s->alpha;
-      const unsigned nb = (unsigned)((s->L.count + 255) / 256);
-      // the balances' coefficients: M (and alpha^2 M^-1 of the four
-      // transverse components) as float32 pairs for float32 fields, M in
-      // float64 for float64 fields
-      if (s->esz == 4) {
-        const bool a2 = c == kHX || c == kHY || c == kEX || c == kEY;
-        rc = dalloc(s, (void**)&s->mp[c], sizeof(float2) * (size_t)s->L.count);
-        if (rc == TETM_OK && a2) rc = dalloc(s, (void**)&s->ap[c], sizeof(float2) * (size_t)s->L.count);
-      } else {
-        rc = dalloc(s, (void**)&s->m_a[c], sizeof(double) * (size_t)s->L.count);
-      }
-      if (rc != TETM_OK) break;
-      if (s->esz == 8)
-        entry_coefs<double><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, 0.0, s->L.count, (double*)s->ua[c], s->m_a[c],
-                                                       nullptr, nullptr);
-      else
-        entry_coefs<float><<<nb, 256, 0, s->stream>>>(s->minv_a[c], sc, s->alpha * s->alpha, s->L.count,
-                                                      (float*)s->ua[c], nullptr, s->mp[c], s->ap[c]);
-      if (cudaGetLastError() != cudaSuccess) rc = TETM_E_CUDA;
-    }
-  }
   if (rc == TETM_OK) rc = rebuild_work(s);
   // (a z-slab keeps the fused sweep, which recomputes its ghost plane's TM half)
   if (rc == TETM_OK && s->esz == 8 && !s->is_slab()) rc = build_band(s);

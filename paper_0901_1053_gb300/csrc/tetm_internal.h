@@ -269,7 +269,7 @@ struct tetm_solver {
   int cur;
   uint8_t* mask;
   double minv_c[6];
-  double* minv_a[6];
+  double* minv_a[6];  // float64 fields, material arrays: M^-1 per entry
   double* m_a[6];  // float64 fields: 1 / minv_a (0 where minv_a is 0), for the balances
   float2* mp[6];   // float32 fields: the same as (hi, lo) float32 pairs
   float2* ap[6];   // float32 fields: alpha^2 minv_a as pairs (kHX, kHY, kEX, kEY)
