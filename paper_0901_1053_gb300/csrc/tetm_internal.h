@@ -368,5 +368,7 @@ void work_list(const tetm_solver* s, int cz, std::vector<int>* list);
 // destroyed on another host thread). Memory is usable on other streams once
 // the allocating stream has reached the allocation.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
+// Copies a caller's (pageable) array to the device, in the order of st
+cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t st);
 void dev_free(void* p, cudaStream_t st);
 }  // namespace tetm
