@@ -22,7 +22,10 @@
 // 4 of 32) cost less than the waits of a lone CTA. A ring for all six inputs
 // instead of register loads, and tensor-map copies into it, were slower (the
 // ring's reads go through the pipe that is full), and so were later loads of
-// e_x, e_y (238 us) and a sweep unrolled by three planes (264 us: code size).
+// e_x, e_y (238 us), a sweep unrolled by three planes (264 us: code size) and
+// one that gathers the transverse wake itself (1.3 us more, the launch 1.5 less
+// only on small grids). With coefficient arrays packed pairs save nothing (192 x
+// 192 x 768, a quarter open: 151.4 against 148.8 us).
 //
 // Only entries that carry a field move through the per-thread loads and
 // stores. Each thread reads the activity bytes of its quad (one 32-bit word
@@ -610,6 +613,10 @@ __global__ void __launch_bounds__(kSThreads, 2)
   Smem& S = *reinterpret_cast<Smem*>(slab_raw);
   const int tid = threadIdx.x;
   const int nitems = a.work ? a.n_work : a.tiles_x * a.tiles_y * a.n_chunks;
+  // every block is resident at once, so the next launch's start (2 us of 205 per
+  // step on 256 x 256 x 1024) hides behind this one's end
+  pdl_trigger();
+  pdl_wait();
 
   // Items in list order: the first per CTA by its index, then (with a
   // schedule counter) whichever item is next when the CTA gets free, fetched
@@ -708,8 +715,7 @@ cudaError_t launch_slab(const StepArgs<float>& a, int* sched, cudaStream_t st) {
   }
   const int items = a.work ? a.n_work : a.tiles_x * a.tiles_y * a.n_chunks;
   if (items <= 0) return cudaSuccess;
-  fused_step_slab<MAT><<<std::min(items, 2 * sms), kSThreads, smem, st>>>(a, sched);
-  return cudaGetLastError();
+  return launch_pdl(fused_step_slab<MAT>, std::min(items, 2 * sms), kSThreads, smem, st, a, sched);
 }
 }  // namespace
 

@@ -62,6 +62,8 @@ __device__ __forceinline__ void transverse_of_step(const StepArgs<T>& a, int k) 
 
 template <typename T>
 __global__ void transverse_after_step(StepArgs<T> a) {
+  pdl_trigger();
+  pdl_wait();
   if (!a.b.obs_on) return;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.L.nz; k += gridDim.x * blockDim.x)
     transverse_of_step(a, k);
@@ -78,8 +80,7 @@ __global__ void transverse_after_batch_step(const BatchMember<T>* members) {
 template <typename T>
 cudaError_t launch_transverse_after_step(const StepArgs<T>& a, cudaStream_t st) {
   const int blocks = std::min(64, (a.L.nz + 127) / 128);
-  transverse_after_step<T><<<blocks, 128, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(transverse_after_step<T>, blocks, 128, 0, st, a);
 }
 
 template <typename T>
