@@ -701,7 +701,8 @@ int do_steps(tetm_solver* s, int n) {
         if constexpr (sizeof(T) == 4) half = s->half && !s->own_shape;
         if (band) {
           if constexpr (sizeof(T) == 8) CK(launch_band_step(a, s->band, s->n_band, s->band_smem, s->stream));
-        } else if (half) {  // with the transverse wake
+          a.b.obs_on = 0;  // the transverse wake is in
+        } else if (half) {
           if constexpr (sizeof(T) == 4) CK(launch_half_step(a, s->half, s->n_half, s->half_run, s->stream));
           a.b.obs_on = 0;
         } else if (warp_shape_ok(s->tile_x, s->tile_y)) {

@@ -23,7 +23,7 @@
 // Per node the operations and their order are those of the other step
 // kernels, so the results are the same bits.
 // Measured per step, warp-tiled sweep (28 x 20 x 32) -> bands: 24 x 24 x 96
-// pipe 1101 -> 14.2 us; collimators 96 x 96 x 384 1189 -> 98 us, 192 x 192 x
+// pipe 1101 -> 14.05 us; collimators 96 x 96 x 384 1189 -> 98 us, 192 x 192 x
 // 384 1200 -> 317 us, 256 x 256 x 1024 2042 -> 1387 us (85% of the float64
 // pipe's rate at 36 instructions per active cell); with coefficient arrays,
 // 96 x 96 x 384, 1151 -> 101 us. 256 threads against 128: the small pipe 14.2
@@ -195,6 +195,15 @@ __global__ void __launch_bounds__(kBThreads, 4) band_te(const StepArgs<double> a
   const double* __restrict__ hy = a.out[kHY] + it.base;
   pdl_trigger();
   pdl_wait();
+  // the transverse wake of the observer line's node, from the old e_x, e_y and
+  // the new h_x, h_y, beside the rest (as a launch of its own behind the step it
+  // made the small pipe 14.2 us instead of 14.05, 17.4 when its start overlapped)
+  const int oi = a.b.obs_i - it.i0, oj = a.b.obs_j - it.j0;
+  if (a.b.obs_on && threadIdx.x == 0 && oi >= 0 && oi < W && oj >= 0 && oj < R) {
+    const long long id = oj * PX + oi;
+    gather_wx(a.b, a.n, it.k, ex[id], hy[id]);
+    gather_wy(a.b, a.n, it.k, ey[id], hx[id]);
+  }
   for (Walk t(R + 2, wx); t.ok(); t.next()) {
     const long long id = (t.r - 1) * PX + t.c - 1;
     const unsigned m = mk[id];
