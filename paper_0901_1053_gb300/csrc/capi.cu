@@ -339,11 +339,16 @@ cudaError_t tetm::dev_alloc(void** p, size_t bytes, cudaStream_t st) {
 // ms to copy on a host that had been busy for a minute, 1.3 ms with the reads
 // before it, which take 0.1 ms (pages of 64 KB).
 cudaError_t tetm::upload(void* dst, const void* src, size_t bytes, cudaStream_t st) {
-  static const long sys = sysconf(_SC_PAGESIZE);
-  const size_t page = sys > 0 ? (size_t)sys : 4096;
-  const volatile unsigned char* p = static_cast<const volatile unsigned char*>(src);
-  for (size_t q = 0; q < bytes; q += page) (void)p[q];
-  if (bytes) (void)p[bytes - 1];
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, src) != cudaSuccess)
+    cudaGetLastError();
+  else if (at.type == cudaMemoryTypeUnregistered) {  // (pinned memory needs none)
+    static const long sys = sysconf(_SC_PAGESIZE);
+    const size_t page = sys > 0 ? (size_t)sys : 4096;
+    const volatile unsigned char* p = static_cast<const volatile unsigned char*>(src);
+    for (size_t q = 0; q < bytes; q += page) (void)p[q];
+    if (bytes) (void)p[bytes - 1];
+  }
   return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
 }
 
@@ -359,11 +364,15 @@ int tile_planes(tetm_solver* s, int tx, int ty, std::vector<uint8_t>* act) {
   const Layout& L = s->L;
   const int tiles_x = (L.nx + tx - 1) / tx, tiles_y = (L.ny + ty - 1) / ty;
   const size_t n = (size_t)tiles_x * tiles_y * L.nz;
+  try {
+    act->resize(n);
+  } catch (const std::bad_alloc&) {
+    return TETM_E_NOMEM;
+  }
   uint8_t* d = nullptr;
   CK(dev_alloc((void**)&d, n, s->stream));
   tile_activity<<<(unsigned)std::min<size_t>((n + 7) / 8, 1u << 16), 256, 0, s->stream>>>(
       s->mask, L, tx, ty, tiles_x, (long long)n, d);
-  act->resize(n);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(act->data(), d, n, cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -452,12 +461,12 @@ int tetm::rebuild_work(tetm_solver* s) {
   const long long tiles = (long long)s->tiles_x * s->tiles_y;
   const int cz_min = s->own_chunk || !s->auto_chunk() ? s->chunk_z : kMinChunk;
   if (tiles * ((L.nz + cz_min - 1) / cz_min) >= (1LL << 31)) return TETM_E_ARG;
+  const int rc = tile_planes(s, s->tile_x, rows, &s->act);
+  if (rc != TETM_OK) return rc;
   if (s->work) {
     dev_free(s->work, s->stream);
     s->work = nullptr;
   }
-  const int rc = tile_planes(s, s->tile_x, rows, &s->act);
-  if (rc != TETM_OK) return rc;
   if (!s->own_chunk) s->chunk_z = s->auto_chunk() ? choose_chunk(s, 1) : kChunk;
   s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
   std::vector<int> list;

@@ -8,7 +8,7 @@
 // 56 x 14 nodes of a run of planes, as short as one, in the shortest case two
 // memory round trips per launch. Two launches move 64 bytes of fields per node
 // instead of 48, which a grid that fits the L2 does not notice; on large ones
-// the sweep is faster (the rule is in choose_half).
+// the sweep is faster (the rule is at build_half in capi.cu).
 // A thread holds two rows of four columns (64 x 16 loaded, 128 threads, four
 // blocks per SM): of the neighbour rows a pair reads, one is its own, so a half
 // exchanges two rows per pair through shared memory, with two block barriers
