@@ -104,9 +104,8 @@ class Autotuner:
         """Shapes (28, ty, cz) whose work-item count fills whole waves of the
         resident warps (16 per SM): for each tile height, the chunk lengths
         around the one that gives one or two full waves; in float32 also slab
-        shapes whose items split evenly over its CTAs (4 to 8 items each):
-        (56, 28, cz), one CTA per SM, or with the material array eps_r
-        (56, 12, cz), two CTAs per SM."""
+        shapes whose items split evenly over its CTAs, two per SM (4 to 8 items
+        each): (56, 28, cz), or (56, 12, cz) with the material array eps_r."""
         from . import tetm
         try:
             import torch
@@ -131,7 +130,7 @@ class Autotuner:
                             best = (eff, c)
                     out.append((28, ty, best[1]))
             if precision == "fp32":
-                ty, ctas = (28, sms) if eps_r is None else (12, 2 * sms)
+                ty, ctas = 28 if eps_r is None else 12, 2 * sms
                 s.set_tiling(56, ty, 32)
                 items32 = s.info()["work_items"]
                 for rounds in range(4, 9):
