@@ -159,7 +159,7 @@ int upload_work(tetm_batch* b) {
 
 template <typename T>
 cudaError_t launch_one(tetm_batch* b) {
-  const int2* work = reinterpret_cast<const int2*>(b->d_wbuf + kHead);
+  int2* work = reinterpret_cast<int2*>(b->d_wbuf + kHead);
   if constexpr (sizeof(T) == 4) {
     if (b->slab)
       return launch_fused_slab_batch((BatchMember<float>*)b->d_members, b->capacity, work, b->d_wbuf,

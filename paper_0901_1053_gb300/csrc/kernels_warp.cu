@@ -882,14 +882,6 @@ cudaError_t launch_fused_warp_batch(const BatchMember<T>* members, int n_members
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_batch_advance(BatchMember<T>* members, int n_members, cudaStream_t st) {
-  batch_advance<T><<<(n_members + 127) / 128, 128, 0, st>>>(members, n_members);
-  return cudaGetLastError();
-}
-template cudaError_t launch_batch_advance<float>(BatchMember<float>*, int, cudaStream_t);
-template cudaError_t launch_batch_advance<double>(BatchMember<double>*, int, cudaStream_t);
-
 template cudaError_t launch_fused_warp_batch<float>(const BatchMember<float>*, int, const int2*, const int*,
                                                     int, int, int, cudaStream_t);
 template cudaError_t launch_fused_warp_batch<double>(const BatchMember<double>*, int, const int2*, const int*,

@@ -144,10 +144,6 @@ bool warp_shape_ok(int tile_x, int tile_y);
 template <typename T>
 cudaError_t launch_fused_warp_batch(const BatchMember<T>* members, int n_members, const int2* work,
                                     const int* n_work, int n_bound, int tile_y, int nz_max, cudaStream_t st);
-// after a batch step: every active member swaps its sets, counts the step
-// and retires at its limit
-template <typename T>
-cudaError_t launch_batch_advance(BatchMember<T>* members, int n_members, cudaStream_t st);
 
 // ---- block-tiled float32 step with a shared-memory ring (kernels_slab.cu):
 // 56 x 12 nodes per item, two CTAs of 256 threads per SM; tetm_set_tiling
@@ -160,8 +156,9 @@ int slab_rows(int tile_x, int tile_y);
 // (work = (member, item) pairs counted at n_work in device memory, at most
 // n_bound; sched as below), the transverse wakes, then the device-side
 // advance of all n_members slots
-cudaError_t launch_fused_slab_batch(BatchMember<float>* members, int n_members, const int2* work,
-                                    const int* n_work, int n_bound, int* sched, int nz_max, cudaStream_t st);
+// (retired members' items leave the list)
+cudaError_t launch_fused_slab_batch(BatchMember<float>* members, int n_members, int2* work, int* n_work, int n_bound,
+                                    int* sched, int nz_max, cudaStream_t st);
 // sched: two ints of device memory, zero before the first launch, that the
 // kernel's dynamic schedule uses and leaves zero (nullptr: static order)
 // (a.co.ua[0] set: the per-entry coefficient arrays of material runs)
