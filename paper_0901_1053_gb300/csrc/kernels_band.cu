@@ -104,11 +104,12 @@ __global__ void __launch_bounds__(kBThreads, 4) band_tm(const StepArgs<double> a
   double* const dex = hya + (R + 1) * wy;
   double* const ezn = dex + (R + 1) * wy;   // rows 0 .. R, columns 0 .. W
   const uint8_t* __restrict__ mk = a.co.mask + it.base;
-  const double* __restrict__ ex = a.in[kEX] + it.base;
-  const double* __restrict__ ey = a.in[kEY] + it.base;
-  const double* __restrict__ ez = a.in[kEZ] + it.base;
-  const double* __restrict__ hx = a.in[kHX] + it.base;
-  const double* __restrict__ hy = a.in[kHY] + it.base;
+  // (no __restrict__: it would let the compiler load a field before pdl_wait)
+  const double* ex = a.in[kEX] + it.base;
+  const double* ey = a.in[kEY] + it.base;
+  const double* ez = a.in[kEZ] + it.base;
+  const double* hx = a.in[kHX] + it.base;
+  const double* hy = a.in[kHY] + it.base;
   pdl_trigger();
   pdl_wait();
   for (Walk t(R + 2, wx); t.ok(); t.next()) {
@@ -188,11 +189,11 @@ __global__ void __launch_bounds__(kBThreads, 4) band_te(const StepArgs<double> a
   double* const dhx = eya + (R + 1) * wy;
   double* const hzn = dhx + (R + 1) * wy;   // rows -1 .. R-1, columns -1 .. W-1
   const uint8_t* __restrict__ mk = a.co.mask + it.base;
-  const double* __restrict__ ex = a.in[kEX] + it.base;
-  const double* __restrict__ ey = a.in[kEY] + it.base;
-  const double* __restrict__ hz = a.in[kHZ] + it.base;
-  const double* __restrict__ hx = a.out[kHX] + it.base;
-  const double* __restrict__ hy = a.out[kHY] + it.base;
+  const double* ex = a.in[kEX] + it.base;
+  const double* ey = a.in[kEY] + it.base;
+  const double* hz = a.in[kHZ] + it.base;
+  const double* hx = a.out[kHX] + it.base;
+  const double* hy = a.out[kHY] + it.base;
   pdl_trigger();
   pdl_wait();
   // the transverse wake of the observer line's node, from the old e_x, e_y and

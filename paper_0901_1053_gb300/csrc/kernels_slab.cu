@@ -130,7 +130,7 @@ __device__ __forceinline__ Q4 ld4_if(const float* p, unsigned c) {
   asm volatile(
       "{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n mov.f32 %0, 0f00000000;\n mov.f32 %1, 0f00000000;\n"
       " mov.f32 %2, 0f00000000;\n mov.f32 %3, 0f00000000;\n"
-      " @q ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];\n}"
+      " @q ld.global.v4.f32 {%0,%1,%2,%3}, [%4];\n}"
       : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
       : "l"(p), "r"(c));
   return r;

@@ -8,7 +8,10 @@
 namespace tetm {
 
 __device__ __forceinline__ unsigned su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-// loads and stores under a predicate, without a branch (zero where not loaded)
+// loads and stores under a predicate, without a branch (zero where not loaded).
+// Only what a solve never changes (the activity bytes) goes through the
+// non-coherent path: a launch that overlaps the one ahead is on the GPU while
+// that one still writes the fields.
 __device__ __forceinline__ unsigned ld_word_if(const uint8_t* p, bool c) {
   unsigned v;
   asm volatile(
@@ -69,7 +72,7 @@ __device__ __forceinline__ P4 ldg_if(const float* p, unsigned c) {
   P4 r;
   asm volatile(
       "{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n mov.b64 %0, 0;\n mov.b64 %1, 0;\n"
-      " @q ld.global.nc.v2.b64 {%0, %1}, [%2];\n}"
+      " @q ld.global.v2.b64 {%0, %1}, [%2];\n}"
       : "=l"(r.a), "=l"(r.b)
       : "l"(p), "r"(c));
   return r;

@@ -1315,8 +1315,8 @@ __global__ void __launch_bounds__(kBandThreads, 4) rz_band_tm(const RzArgs<T> a,
   T* const hra = der + P * w2;                      // columns 0 .. W
   T* const dep = hra + P * w1;
   T* const ezn = dep + P * w1;
-  const T* __restrict__ in = a.in + b.f;
-  T* __restrict__ out = a.out + b.f;
+  const T* in = a.in + b.f;  // (no __restrict__: it would let the compiler load a field before pdl_wait)
+  T* out = a.out + b.f;
   tetm::pdl_trigger();
   tetm::pdl_wait();
   for (RzWalk t(P, w2); t.ok(); t.next()) {
@@ -1400,8 +1400,8 @@ __global__ void __launch_bounds__(kBandThreads, 4) rz_band_te(const RzArgs<T> a,
   const RzBand<T> b = rz_band(a, items);
   const long long PR = a.L.pr, RS = 6 * PR;
   const int P = b.planes, W = b.w, w2 = W + 2, w1 = W + 1;
-  const T* __restrict__ in = a.in + b.f;
-  T* __restrict__ out = a.out + b.f;  // h_phi, h_r as rz_band_tm left them
+  const T* in = a.in + b.f;
+  T* out = a.out + b.f;  // h_phi, h_r as rz_band_tm left them
   tetm::pdl_trigger();
   tetm::pdl_wait();
   if (b.tm_only) {

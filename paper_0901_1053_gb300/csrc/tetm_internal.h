@@ -328,7 +328,10 @@ namespace tetm {
 // A launch that may begin before the kernel ahead of it in the stream has
 // ended: the kernel calls pdl_wait() before it reads or writes anything a
 // kernel ahead may write or read (what a solve never changes, its work list
-// and activity bytes, may be read before). pdl_trigger() in a kernel lets the
+// and activity bytes, may be read before). It is on the GPU while the kernel
+// ahead still writes, so it loads fields by plain loads: the non-coherent path
+// (ld.global.nc, or what const __restrict__ pointers license) is for data that
+// no one writes as long as the kernel lives. pdl_trigger() in a kernel lets the
 // next such launch begin; it is called once every block runs, so the next
 // launch's blocks never take the place of blocks still to start.
 template <typename... P, typename... A>
