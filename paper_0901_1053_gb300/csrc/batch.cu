@@ -310,7 +310,7 @@ int check_member(const tetm_batch* b, const tetm_solver* s) {
 }
 
 template <typename T>
-int write_member(tetm_batch* b, int i, tetm_solver* s) {
+int write_member(tetm_batch* b, int i, tetm_solver* s) try {
   BatchMember<T> m;
   memset(&m, 0, sizeof(m));
   m.a = step_args<T>(s, true);
@@ -320,7 +320,7 @@ int write_member(tetm_batch* b, int i, tetm_solver* s) {
   std::vector<int>& items = b->items[(size_t)i];
   items = s->work_host;
   if (b->slab && !s->own_chunk && s->auto_chunk()) {
-    m.a.chunk_z = choose_chunk(s, b->capacity);
+    m.a.chunk_z = choose_chunk(s->act, s->L.nz, b->capacity);
     m.a.n_chunks = (s->L.nz + m.a.chunk_z - 1) / m.a.chunk_z;
     work_list(s, m.a.chunk_z, &items);
   }
@@ -328,6 +328,8 @@ int write_member(tetm_batch* b, int i, tetm_solver* s) {
   m.active = s->step < b->limit[(size_t)i] ? 1 : 0;
   m.cur = s->cur;
   return stage_copy(b, (char*)b->d_members + sizeof(BatchMember<T>) * (size_t)i, &m, sizeof(m));
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
 }
 
 int add_member(tetm_batch* b, tetm_solver* s, long long limit, int* slot_out) {
@@ -337,9 +339,7 @@ int add_member(tetm_batch* b, tetm_solver* s, long long limit, int* slot_out) {
   while (i < b->capacity && b->slot[(size_t)i]) ++i;
   if (i == b->capacity) return TETM_E_STATE;
   if (s->tile_x != b->tile_x || s->tile_y != b->tile_y || s->work_dirty) {
-    s->tile_x = b->tile_x;
-    s->tile_y = b->tile_y;
-    rc = rebuild_work(s);
+    rc = reshape(s, b->tile_x, b->tile_y, s->chunk_z, s->own_shape, s->own_chunk);
     if (rc != TETM_OK) return rc;
   }
   // the batch's stream first waits for the work queued on the member's own

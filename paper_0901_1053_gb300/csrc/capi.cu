@@ -264,6 +264,7 @@ double phi(double x) { return 0.5 * erfc(-x / sqrt(2.0)); }
 namespace {
 
 int cuda_fail(cudaError_t e) {
+  cudaGetLastError();  // answered here: the next launch's check must not see it again
   if (e == cudaErrorMemoryAllocation) return TETM_E_NOMEM;
   return TETM_E_CUDA;
 }
@@ -433,12 +434,12 @@ void tetm::work_list(const tetm_solver* s, int cz, std::vector<int>* list) { ite
 // the last one counts by half: items * share / slots + 1/2 on average, at least
 // one, and no more than kChunk planes, since the others may leave early (a batch
 // of 16: 406 ms at 20 to 32 planes, 441 at 8, 423 at 64).
-int tetm::choose_chunk(const tetm_solver* s, int share, double* out) {
-  const int nz = s->L.nz, sms = sm_count();
+int tetm::choose_chunk(const std::vector<uint8_t>& act, int nz, int share, double* out) {
+  const int sms = sm_count();
   const int top = std::min(share == 1 ? kMaxChunk : kChunk, std::max(nz, kMinChunk));
   if (sms < 1) return kChunk;
   const double slots = 2.0 * sms;
-  const std::vector<long long> items = count_items(s->act, nz, kMinChunk, top);
+  const std::vector<long long> items = count_items(act, nz, kMinChunk, top);
   int best = kMinChunk;
   double least = 0.0;
   for (int cz = kMinChunk; cz <= top; ++cz) {
@@ -453,54 +454,87 @@ int tetm::choose_chunk(const tetm_solver* s, int share, double* out) {
   return best;
 }
 
-int tetm::rebuild_work(tetm_solver* s) {
+// All of it is made before anything of the solve changes: a rebuild that fails
+// leaves the shape, the item list and the partials as they were, fit for each
+// other (a list read under another tile shape would walk past the grid).
+int tetm::rebuild_work(tetm_solver* s) try {
   const Layout& L = s->L;
-  s->tiles_x = (L.nx + s->tile_x - 1) / s->tile_x;
   const int rows = slab_rows(s->tile_x, s->tile_y);
-  s->tiles_y = (L.ny + rows - 1) / rows;
-  const long long tiles = (long long)s->tiles_x * s->tiles_y;
+  const int tiles_x = (L.nx + s->tile_x - 1) / s->tile_x, tiles_y = (L.ny + rows - 1) / rows;
+  const long long tiles = (long long)tiles_x * tiles_y;
   const int cz_min = s->own_chunk || !s->auto_chunk() ? s->chunk_z : kMinChunk;
   if (tiles * ((L.nz + cz_min - 1) / cz_min) >= (1LL << 31)) return TETM_E_ARG;
-  const int rc = tile_planes(s, s->tile_x, rows, &s->act);
+  std::vector<uint8_t> act;
+  const int rc = tile_planes(s, s->tile_x, rows, &act);
   if (rc != TETM_OK) return rc;
-  if (s->work) {
-    dev_free(s->work, s->stream);
-    s->work = nullptr;
-  }
-  if (!s->own_chunk) s->chunk_z = s->auto_chunk() ? choose_chunk(s, 1) : kChunk;
-  s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
+  const int cz = s->own_chunk ? s->chunk_z : s->auto_chunk() ? choose_chunk(act, L.nz, 1) : kChunk;
   std::vector<int> list;
-  work_list(s, s->chunk_z, &list);
-  s->n_work = (int)list.size();
-  s->work_host = list;
-  if (3 * s->n_work > s->diag.cap) {  // balance reductions keep three partials per work item
+  items_of(act, L.nz, cz, &list);
+  int* work = nullptr;
+  double* part = nullptr;
+  const int cap = std::max(2048, 3 * (int)list.size());  // balance reductions keep three partials per work item
+  cudaError_t e = cudaSuccess;
+  if (cap > s->diag.cap) e = dev_alloc((void**)&part, sizeof(double) * (size_t)cap, s->stream);
+  if (e == cudaSuccess && !list.empty()) {
+    e = dev_alloc((void**)&work, sizeof(int) * list.size(), s->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(work, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  }
+  if (e != cudaSuccess) {
+    dev_free(work, s->stream);
+    dev_free(part, s->stream);
+    return cuda_fail(e);
+  }
+  if (part) {
     dev_free(s->diag.part, s->stream);
-    s->diag.part = nullptr;
-    s->diag.cap = 0;
-    const int cap = std::max(2048, 3 * s->n_work);
-    CK(dev_alloc((void**)&s->diag.part, sizeof(double) * (size_t)cap, s->stream));
+    s->diag.part = part;
     s->diag.cap = cap;
   }
-  if (!list.empty()) {
-    CK(dev_alloc((void**)&s->work, sizeof(int) * list.size(), s->stream));
-    CK(cudaMemcpyAsync(s->work, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice,
-                       s->stream));
-    CK(cudaStreamSynchronize(s->stream));
-  }
+  dev_free(s->work, s->stream);
+  s->work = work;
+  s->tiles_x = tiles_x;
+  s->tiles_y = tiles_y;
+  s->chunk_z = cz;
+  s->n_chunks = (L.nz + cz - 1) / cz;
+  s->n_work = (int)list.size();
+  s->work_host = std::move(list);
+  s->act = std::move(act);
   s->work_dirty = false;
   return TETM_OK;
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
+}
+
+int tetm::reshape(tetm_solver* s, int tile_x, int tile_y, int chunk_z, bool own_shape, bool own_chunk) {
+  const int x = s->tile_x, y = s->tile_y, z = s->chunk_z;
+  const bool os = s->own_shape, oc = s->own_chunk;
+  s->tile_x = tile_x;
+  s->tile_y = tile_y;
+  s->chunk_z = chunk_z;
+  s->own_shape = own_shape;
+  s->own_chunk = own_chunk;
+  const int rc = rebuild_work(s);
+  if (rc != TETM_OK) {
+    s->tile_x = x;
+    s->tile_y = y;
+    s->chunk_z = z;
+    s->own_shape = os;
+    s->own_chunk = oc;
+  }
+  return rc;
 }
 
 namespace {
 
 // Work items of the float64 band kernels: the column hulls of the active
 // entries per (plane, band) from the device, the list from them.
-int build_band(tetm_solver* s) {
+int build_band(tetm_solver* s) try {
   const int rows = band_rows(s->active_cells);
   const size_t n = (size_t)((s->L.ny + rows - 1) / rows) * (size_t)s->L.nz;
+  std::vector<int2> h(n);
   int2* d = nullptr;
   CK(dev_alloc((void**)&d, sizeof(int2) * n, s->stream));
-  std::vector<int2> h(n);
   cudaError_t e = launch_band_hulls(s->mask, s->L, rows, d, s->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(int2) * n, cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -515,6 +549,8 @@ int build_band(tetm_solver* s) {
   CK(cudaMemcpyAsync(s->band, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   return TETM_OK;
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
 }
 
 // Work items of the half-step kernels, where they are the faster float32 step
@@ -526,11 +562,11 @@ int build_band(tetm_solver* s) {
 // 14.4 | 10.8 at 3.7e5, 20.5 | 14.7 at 6.3e5; beyond, the halves' fuller SMs and
 // 64 bytes per node cost more: 20.5 | 21.2 at 8.7e5, 28.7 | 31.8 at 1.4e6.
 constexpr long long kHalfCells = 3LL << 18;
-int build_half(tetm_solver* s) {
+int build_half(tetm_solver* s) try {
   const int nz = s->L.nz, sms = sm_count();
   if (sms < 1 || s->n_work == 0 || s->active_cells > kHalfCells) return TETM_OK;
   double sweep = 0.0;
-  choose_chunk(s, 1, &sweep);
+  choose_chunk(s->act, nz, 1, &sweep);
   const double slots = (double)kHalfBlocks * sms;
   std::vector<uint8_t> act;
   int rc = tile_planes(s, kHalfX, kHalfY, &act);
@@ -551,6 +587,8 @@ int build_half(tetm_solver* s) {
   CK(cudaMemcpyAsync(s->half, list.data(), sizeof(int) * list.size(), cudaMemcpyHostToDevice, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   return TETM_OK;
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
 }
 
 }  // namespace
@@ -1144,9 +1182,7 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   if (s->scheme == TETM_SCHEME_YEE) {  // Yee's fused kernel has one tile shape
     if (tx != s->tile_x || ty != s->tile_y) return TETM_E_UNSUPPORTED;
     if (cz < 4) return TETM_E_ARG;
-    if (chunk_z) s->own_chunk = true;
-    s->chunk_z = cz;
-    return rebuild_work(s);
+    return reshape(s, tx, ty, cz, s->own_shape, s->own_chunk || chunk_z);
   }
   const bool slab_u = slab_shape_ok(tx, ty, false), slab_m = slab_shape_ok(tx, ty, true);
   if ((!fused_shape_ok(tx, ty) && !warp_shape_ok(tx, ty) && !slab_u && !slab_m) || cz < 4)
@@ -1159,13 +1195,13 @@ int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chun
   // the slab kernel is float32 only
   if ((slab_u || slab_m) && s->esz != 4) return TETM_E_UNSUPPORTED;
   if (s->kernel == TETM_KERNEL_TWOSTEP && !fused2_shape_ok(tx, ty)) return TETM_E_UNSUPPORTED;
-  if (tile_x || tile_y || chunk_z) s->own_shape = true;
-  if (chunk_z) s->own_chunk = true;
-  if (tx == s->tile_x && ty == s->tile_y && cz == s->chunk_z && s->work) return TETM_OK;
-  s->tile_x = tx;
-  s->tile_y = ty;
-  s->chunk_z = cz;
-  return rebuild_work(s);
+  const bool own_shape = s->own_shape || tile_x || tile_y || chunk_z, own_chunk = s->own_chunk || chunk_z;
+  if (tx == s->tile_x && ty == s->tile_y && cz == s->chunk_z && s->work) {
+    s->own_shape = own_shape;
+    s->own_chunk = own_chunk;
+    return TETM_OK;
+  }
+  return reshape(s, tx, ty, cz, own_shape, own_chunk);
 }
 
 int tetm_set_scheme(tetm_solver* s, int32_t scheme) {
@@ -1173,17 +1209,19 @@ int tetm_set_scheme(tetm_solver* s, int32_t scheme) {
   if (scheme == s->scheme) return TETM_OK;
   if (s->is_slab() || s->kernel == TETM_KERNEL_TWOSTEP) return TETM_E_UNSUPPORTED;
   if (s->step != 0 || s->bunch || s->in_batch || s->bal_every > 0) return TETM_E_STATE;
+  int tx, ty;
   if (scheme == TETM_SCHEME_YEE) {
     const double dx = s->g.dx, dy = s->g.dy, dz = s->g.dz;
     const double lim = 1.0 / sqrt(1.0 / (dx * dx) + 1.0 / (dy * dy) + 1.0 / (dz * dz));  // Eq. (8)
     if (s->g.cdt > lim * (1.0 + 1e-12)) return TETM_E_UNSTABLE;
-    yee_shape((int)s->esz, &s->tile_x, &s->tile_y);
+    yee_shape((int)s->esz, &tx, &ty);
   } else {  // the TE/TM scheme's default work shape
-    s->tile_x = s->esz == 4 ? 56 : 28;
-    s->tile_y = s->esz == 4 ? (s->uniform ? 28 : 12) : 20;
+    tx = s->esz == 4 ? 56 : 28;
+    ty = s->esz == 4 ? (s->uniform ? 28 : 12) : 20;
   }
-  s->scheme = scheme;
-  return rebuild_work(s);
+  const int rc = reshape(s, tx, ty, s->chunk_z, s->own_shape, s->own_chunk);
+  if (rc == TETM_OK) s->scheme = scheme;
+  return rc;
 }
 
 int tetm_set_bunch(tetm_solver* s, double sigma_z, double charge, int32_t i0, int32_t j0) {

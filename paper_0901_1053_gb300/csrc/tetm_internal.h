@@ -355,11 +355,14 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 template <typename T>
 StepArgs<T> step_args(tetm_solver* s, bool fused);
 // (re)build the list of (tile, chunk) work items that own a field-carrying cell
+// (a failure changes nothing)
 int rebuild_work(tetm_solver* s);
+// takes another work shape: the solve's shape, list and partials as a whole, or none of them
+int reshape(tetm_solver* s, int tile_x, int tile_y, int chunk_z, bool own_shape, bool own_chunk);
 constexpr int kChunk = 32, kMinChunk = 4, kMaxChunk = 64;  // planes per work item: set ones start at kMinChunk
 // the slab kernel's planes per item for one of `share` solves that step
-// together, and the items of chunks of cz planes (both from s->act)
-int choose_chunk(const tetm_solver* s, int share, double* cost = nullptr);
+// together (act: per tile and plane, as tetm_solver::act), and the items of chunks of cz planes
+int choose_chunk(const std::vector<uint8_t>& act, int nz, int share, double* cost = nullptr);
 void work_list(const tetm_solver* s, int cz, std::vector<int>* list);
 // Device memory of solves and batches comes from one stream-ordered pool per
 // device: allocation and release are queued on the given stream, so neither
