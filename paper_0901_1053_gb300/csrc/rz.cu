@@ -2380,13 +2380,13 @@ int rz_occupancy(tetm_rz* s) {
   return TETM_OK;
 }
 
-int rz_rebuild_work(tetm_rz* s) {
+// All of it is made before anything of the solve changes: a rebuild that fails
+// leaves the windows and the item list as they were, fit for each other.
+int rz_rebuild_work(tetm_rz* s) try {
   const RzLayout& L = s->L;
   const int tw = rz_kernel(s) == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile;
-  s->tile_w = tw;
-  s->tiles = (L.nr + 1 + tw - 1) / tw;
-  s->n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
-  const int nf = s->tiles * s->n_chunks;
+  const int tiles = (L.nr + 1 + tw - 1) / tw, n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
+  const int nf = tiles * n_chunks;
   if (nf > s->flags_cap) {
     cudaFree(s->flags);
     s->flags = nullptr;
@@ -2395,47 +2395,76 @@ int rz_rebuild_work(tetm_rz* s) {
     if (e != cudaSuccess) return rz_fail(e);
     s->flags_cap = nf;
   }
-  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, L, s->tiles, tw, s->chunk_z,
-                                                      s->n_chunks, s->flags);
+  std::vector<int> fl((size_t)nf);
+  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, L, tiles, tw, s->chunk_z, n_chunks, s->flags);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rz_fail(e);
-  std::vector<int> fl((size_t)nf);
   e = cudaMemcpyAsync(fl.data(), s->flags, sizeof(int) * (size_t)nf, cudaMemcpyDeviceToHost, s->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   if (e != cudaSuccess) return rz_fail(e);
-  std::vector<int> w;
+  std::vector<int> w, first((size_t)n_chunks + 1, 0);
   long long processed = 0;
-  s->chunk_first.assign((size_t)s->n_chunks + 1, 0);
   for (int q = 0; q < nf; ++q) {
-    if (q % s->tiles == 0) s->chunk_first[(size_t)(q / s->tiles)] = (int)w.size();
+    if (q % tiles == 0) first[(size_t)(q / tiles)] = (int)w.size();
     if (!fl[(size_t)q]) continue;
     w.push_back(q);
-    const int tile = q % s->tiles, chunk = q / s->tiles;
+    const int tile = q % tiles, chunk = q / tiles;
     const int width = std::min(tw, L.nr + 1 - tile * tw);
     const int planes = std::min(s->chunk_z, L.nz - chunk * s->chunk_z);
     processed += (long long)width * planes;
   }
-  cudaFree(s->work);
-  s->work = nullptr;
+  first[(size_t)n_chunks] = (int)w.size();
+  int* work = nullptr;
   if (!w.empty()) {
-    e = cudaMalloc(&s->work, sizeof(int) * w.size());
-    if (e != cudaSuccess) return rz_fail(e);
-    e = cudaMemcpy(s->work, w.data(), sizeof(int) * w.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return rz_fail(e);
+    e = cudaMalloc(&work, sizeof(int) * w.size());
+    if (e == cudaSuccess) e = cudaMemcpy(work, w.data(), sizeof(int) * w.size(), cudaMemcpyHostToDevice);
   }
-  if (s->esz == 4 && tw == kTile2 && !s->changes) {  // once: they depend on the geometry only
+  if (e == cudaSuccess && s->esz == 4 && tw == kTile2 && !s->changes) {  // once: they depend on the geometry only
     s->change_words = (int)((L.rows + 31) / 32);
-    const long long warps = (long long)s->tiles * s->change_words;
+    const long long warps = (long long)tiles * s->change_words;
     e = cudaMalloc(&s->changes, sizeof(unsigned) * (size_t)warps);
-    if (e != cudaSuccess) return rz_fail(e);
-    rz_mask_changes<<<(unsigned)((warps + 7) / 8), 256, 0, s->st>>>(s->mask, L, s->tiles, s->change_words, s->changes);
-    if ((e = cudaGetLastError()) != cudaSuccess) return rz_fail(e);
+    if (e == cudaSuccess) {
+      rz_mask_changes<<<(unsigned)((warps + 7) / 8), 256, 0, s->st>>>(s->mask, L, tiles, s->change_words, s->changes);
+      if ((e = cudaGetLastError()) != cudaSuccess) {
+        cudaFree(s->changes);
+        s->changes = nullptr;
+      }
+    }
   }
+  if (e != cudaSuccess) {
+    cudaFree(work);
+    return rz_fail(e);
+  }
+  cudaFree(s->work);
+  s->work = work;
+  s->tile_w = tw;
+  s->tiles = tiles;
+  s->n_chunks = n_chunks;
+  s->chunk_first = std::move(first);
   s->n_work = (int)w.size();
-  s->chunk_first[(size_t)s->n_chunks] = s->n_work;
   s->processed = processed * s->n_modes;
   s->work_dirty = false;
   return TETM_OK;
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
+}
+
+// Takes the caller's kernel and chunk length, or (on a failure) nothing of them.
+int rz_reshape(tetm_rz* s, int kernel, int chunk_z, bool retile) {
+  const int k = s->kernel, z = s->chunk_z, resident = s->resident;
+  const bool own = s->own_shape;
+  s->kernel = kernel;
+  s->chunk_z = chunk_z;
+  s->own_shape = true;
+  int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
+  if (rc == TETM_OK && retile) rc = rz_rebuild_work(s);
+  if (rc != TETM_OK) {
+    s->kernel = k;
+    s->chunk_z = z;
+    s->own_shape = own;
+    s->resident = resident;
+  }
+  return rc;
 }
 
 // Planes per work item until a length is chosen: about four items per resident
@@ -3167,15 +3196,7 @@ int tetm_rz_set_fields(tetm_rz* s, int32_t mode, int32_t comp, const double* in)
 
 int tetm_rz_set_tiling(tetm_rz* s, int32_t chunk_z) {
   if (!s || chunk_z < 4 || chunk_z > (1 << 20)) return TETM_E_ARG;
-  s->chunk_z = chunk_z;
-  const bool first = !s->own_shape;
-  s->own_shape = true;
-  s->work_dirty = true;
-  if (first) {  // the kernel may change with it
-    const int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
-    if (rc != TETM_OK) return rc;
-  }
-  return rz_rebuild_work(s);
+  return rz_reshape(s, s->kernel, chunk_z, true);  // (the kernel may change with the first one)
 }
 
 int tetm_rz_set_kernel(tetm_rz* s, int32_t kernel) {
@@ -3184,12 +3205,7 @@ int tetm_rz_set_kernel(tetm_rz* s, int32_t kernel) {
     return TETM_E_ARG;
   if (s->mat && kernel != TETM_RZ_KERNEL_REGISTER) return TETM_E_UNSUPPORTED;  // per-plane coefficients
   const bool retile = !s->own_shape || (kernel == TETM_RZ_KERNEL_BULK2) != (s->kernel == TETM_RZ_KERNEL_BULK2);
-  s->kernel = kernel;
-  if (!s->own_shape) s->chunk_z = kDefaultChunk;
-  s->own_shape = true;
-  int rc = s->esz == 8 ? rz_occupancy<double>(s) : rz_occupancy<float>(s);
-  if (rc == TETM_OK && retile) rc = rz_rebuild_work(s);
-  return rc;
+  return rz_reshape(s, kernel, s->own_shape ? s->chunk_z : kDefaultChunk, retile);
 }
 
 int tetm_rz_set_stream(tetm_rz* s, void* cuda_stream) {

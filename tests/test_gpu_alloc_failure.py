@@ -127,7 +127,96 @@ print("all kept")
 """
 
 
-@pytest.mark.parametrize("source,shim,child", [("capi.cu", SHIM, CHILD)], ids=["cartesian"])
+RZ_SHIM = """
+#include <cuda_runtime.h>
+extern "C" { __attribute__((visibility("default"))) int fail_alloc_at = 0; }  // 1: the next one, 0: none
+template <typename P>
+static inline cudaError_t alloc_or_fail(P* p, size_t bytes) {
+  if (fail_alloc_at > 0 && --fail_alloc_at == 0) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+#define cudaMalloc alloc_or_fail
+"""
+
+RZ_CHILD = """
+import ctypes, sys
+sys.path.insert(0, %(root)r)
+from paper_0901_1053_gb300 import build
+build.library_path = lambda: %(lib)r
+import numpy as np
+from paper_0901_1053_gb300 import tetm, workloads as wl
+
+fail = ctypes.c_int.in_dll(tetm.lib, "fail_alloc_at")
+SHAPE = ("chunk_z", "work_items", "processed_cells", "resident_warps", "kernel")
+NR, NZ = 130, 90
+pec = wl.cavity_chain_rz(NR, NZ, 0, 2).pec
+
+def solver(precision):
+    s = tetm.RzSolver(NR, NZ, 0, 1, 1e-3, 1e-3, 1e-3, precision, pec=pec)
+    rng = np.random.default_rng(3)
+    for m in (0, 1):
+        for c in range(6):
+            s.set(m, c, rng.standard_normal(s.shape))
+    return s
+
+def shape(s):
+    return [s.info()[k] for k in SHAPE]
+
+def refused(call, s):
+    before, n = shape(s), 0
+    while True:
+        n += 1
+        fail.value = n
+        try:
+            call()
+        except tetm.TetmError as e:
+            assert e.code == tetm.TETM_E_NOMEM, e.code
+            assert shape(s) == before, (shape(s), before)
+        else:
+            assert fail.value > 0
+            fail.value = 0
+            return n - 1
+
+def same(a, b):
+    for m in (0, 1):
+        for c in range(6):
+            assert np.array_equal(a.get(m, c), b.get(m, c))
+
+for precision in ("fp32", "fp64"):
+    s, want = solver(precision), solver(precision)
+    n0 = shape(s)
+    fail.value = 1
+    try:
+        s.set_kernel("bulk")
+        raise SystemExit("accepted without memory")
+    except tetm.TetmError:
+        assert shape(s) == n0, (shape(s), n0)
+    s.step(3)                            # on the library's choice
+    want.step(3)
+    same(s, want)
+    for kernel, chunk in (("bulk", 5), ("bulk2", 4), ("register", 90)):
+        assert refused(lambda: s.set_kernel(kernel), s) <= 2
+        assert refused(lambda: s.set_tiling(chunk), s) >= 1
+        s.step(3)
+        want.step(3)
+        same(s, want)
+    s.close()
+    want.close()
+    for n in range(1, 100):              # a solve that cannot be made: an error, whatever the allocation
+        fail.value = n
+        try:
+            solver(precision).close()
+        except tetm.TetmError:
+            continue
+        break
+    assert 8 < n < 99 and fail.value > 0, n
+    fail.value = 0
+print("all kept")
+"""
+
+
+@pytest.mark.parametrize("source,shim,child", [("capi.cu", SHIM, CHILD), ("rz.cu", RZ_SHIM, RZ_CHILD)],
+                         ids=["cartesian", "rz"])
 def test_a_failed_change_of_shape_changes_nothing(tmp_path, source, shim, child):
     import __graft_entry__
     __graft_entry__.build()
