@@ -2425,7 +2425,10 @@ int rz_rebuild_work(tetm_rz* s) try {
     e = cudaMalloc(&s->changes, sizeof(unsigned) * (size_t)warps);
     if (e == cudaSuccess) {
       rz_mask_changes<<<(unsigned)((warps + 7) / 8), 256, 0, s->st>>>(s->mask, L, tiles, s->change_words, s->changes);
-      if ((e = cudaGetLastError()) != cudaSuccess) {
+      e = cudaGetLastError();
+      // (the caller may step on another stream next: tetm_rz_set_stream)
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+      if (e != cudaSuccess) {
         cudaFree(s->changes);
         s->changes = nullptr;
       }
