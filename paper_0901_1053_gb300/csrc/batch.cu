@@ -315,12 +315,12 @@ int write_member(tetm_batch* b, int i, tetm_solver* s) try {
   memset(&m, 0, sizeof(m));
   m.a = step_args<T>(s, true);
   m.a.work = nullptr;  // the batch's combined list is used instead
-  // in it the member's items have the length that suits a share of the GPU
-  // (choose_chunk), unless the caller set one; its own list stays as it is
+  // in it the member's items have the length the caller set, or else the one
+  // that suits a share of the GPU (choose_chunk); its own list stays as it is
   std::vector<int>& items = b->items[(size_t)i];
   items = s->work_host;
-  if (b->slab && !s->own_chunk && s->auto_chunk()) {
-    m.a.chunk_z = choose_chunk(s->act, s->L.nz, b->capacity);
+  if (b->slab && s->auto_chunk()) {
+    m.a.chunk_z = s->own_chunk ? s->chunk_z : choose_chunk(s->act, s->L.nz, b->capacity);
     m.a.n_chunks = (s->L.nz + m.a.chunk_z - 1) / m.a.chunk_z;
     work_list(s, m.a.chunk_z, &items);
   }

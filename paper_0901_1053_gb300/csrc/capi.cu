@@ -454,6 +454,28 @@ int tetm::choose_chunk(const std::vector<uint8_t>& act, int nz, int share, doubl
   return best;
 }
 
+namespace {
+
+// Planes per work item for a chunk the caller set on the shape 56 x 28, whose
+// items own 12 rows: the set number, or, where that leaves the last round of
+// the GPU's slots so empty that the step takes a tenth longer by the cost of
+// choose_chunk, the best one of no less than half of it. The same chunk makes
+// more than twice the items it made at 28 rows, and one round of those can
+// become two with the second nearly empty.
+int fit_chunk(const std::vector<uint8_t>& act, int nz, int cz) {
+  const int sms = sm_count(), hi = std::min(cz, nz), lo = std::max(kMinChunk, (hi + 1) / 2);
+  if (sms < 1 || lo >= hi) return cz;
+  const double slots = 2.0 * sms;
+  const std::vector<long long> items = count_items(act, nz, lo, hi);
+  auto cost = [&](int c) { return ceil((double)items[(size_t)c] / slots) * (c + 2); };
+  int best = hi;
+  for (int c = hi - 1; c >= lo; --c)
+    if (cost(c) < cost(best)) best = c;
+  return cost(best) < 0.9 * cost(hi) ? best : cz;
+}
+
+}  // namespace
+
 // All of it is made before anything of the solve changes: a rebuild that fails
 // leaves the shape, the item list and the partials as they were, fit for each
 // other (a list read under another tile shape would walk past the grid).
@@ -462,14 +484,15 @@ int tetm::rebuild_work(tetm_solver* s) try {
   const int rows = slab_rows(s->tile_x, s->tile_y);
   const int tiles_x = (L.nx + s->tile_x - 1) / s->tile_x, tiles_y = (L.ny + rows - 1) / rows;
   const long long tiles = (long long)tiles_x * tiles_y;
-  const int cz_min = s->own_chunk || !s->auto_chunk() ? s->chunk_z : kMinChunk;
+  const int cz_min = s->auto_chunk() ? kMinChunk : s->chunk_z;
   if (tiles * ((L.nz + cz_min - 1) / cz_min) >= (1LL << 31)) return TETM_E_ARG;
   std::vector<uint8_t> act;
   const int rc = tile_planes(s, s->tile_x, rows, &act);
   if (rc != TETM_OK) return rc;
   const int cz = s->own_chunk ? s->chunk_z : s->auto_chunk() ? choose_chunk(act, L.nz, 1) : kChunk;
+  const int item_z = s->own_chunk && rows != s->tile_y ? fit_chunk(act, L.nz, cz) : cz;
   std::vector<int> list;
-  items_of(act, L.nz, cz, &list);
+  items_of(act, L.nz, item_z, &list);
   int* work = nullptr;
   double* part = nullptr;
   const int cap = std::max(2048, 3 * (int)list.size());  // balance reductions keep three partials per work item
@@ -496,7 +519,8 @@ int tetm::rebuild_work(tetm_solver* s) try {
   s->tiles_x = tiles_x;
   s->tiles_y = tiles_y;
   s->chunk_z = cz;
-  s->n_chunks = (L.nz + cz - 1) / cz;
+  s->item_z = item_z;
+  s->n_chunks = (L.nz + item_z - 1) / item_z;
   s->n_work = (int)list.size();
   s->work_host = std::move(list);
   s->act = std::move(act);
@@ -634,7 +658,7 @@ StepArgs<T> tetm::step_args(tetm_solver* s, bool fused) {
   }
   a.tiles_x = s->tiles_x;
   a.tiles_y = s->tiles_y;
-  a.chunk_z = s->chunk_z;
+  a.chunk_z = s->item_z;
   a.n_chunks = s->n_chunks;
   a.work = s->work;
   a.n_work = s->n_work;
@@ -654,7 +678,7 @@ WorkView work_view(const tetm_solver* s) {
   v.n_items = s->n_work;
   v.tile_x = s->tile_x;
   v.tile_y = slab_rows(s->tile_x, s->tile_y);
-  v.chunk_z = s->chunk_z;
+  v.chunk_z = s->item_z;
   v.tiles_x = s->tiles_x;
   v.tiles_y = s->tiles_y;
   return v;
@@ -1510,7 +1534,7 @@ int tetm_get_info(tetm_solver* s, tetm_info* info) {
   info->step = s->step;
   info->device_bytes = s->device_bytes;
   info->active_cells = s->active_cells;
-  info->processed_cells = (long long)s->n_work * s->tile_x * slab_rows(s->tile_x, s->tile_y) * s->chunk_z;
+  info->processed_cells = (long long)s->n_work * s->tile_x * slab_rows(s->tile_x, s->tile_y) * s->item_z;
   info->kernel = s->kernel;
   info->precision = s->g.precision;
   info->tile_x = s->tile_x;

@@ -278,6 +278,7 @@ struct tetm_solver {
   int scheme;     // TETM_SCHEME_*
   int kernel;
   int tile_x, tile_y, chunk_z;
+  int item_z;                  // planes of an item of the list: chunk_z, or fewer (fit_chunk in capi.cu)
   int* sched;                    // the slab kernel's schedule counters (two ints)
   int tiles_x, tiles_y, n_chunks;
   int* work;
