@@ -56,10 +56,25 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// The wake sample of a warp's bunch line node: add_wake's addition (RED), or the
+// same as a load, an addition and a store, the same bits. Around the one
+// addition the row loops are compiled into slower ones in float32 (us per step:
+// 335 | 326 with 28 x 20 x 32 on 48 x 48 x 192, 555 | 546 with 28 x 28 x 32 on
+// 118 x 131 x 603) and in float64 batches (1143 | 1132 on eight of 48 x 48 x
+// 192); alone in float64 it is the faster (1120 | 1190 on 128 x 128 x 512).
+template <bool RED, typename T>
+__device__ __forceinline__ void warp_wake(const BunchDev<T>& b, long long m, T ez) {
+  if constexpr (RED) {
+    add_wake(b, m, ez);
+  } else {
+    if (m >= b.m_min && m <= b.m_max) b.W[m - b.m_min] -= __dmul_rn((double)ez, b.inv_q);
+  }
+}
+
 constexpr int kDepth = 8;   // rows of loads in flight ahead of the sweep
 constexpr int kArrs = 8;    // ez hx hy hz (plane k), ex ey (plane k), ex ey (plane k+1)
 
-template <typename T, int TY>
+template <typename T, int TY, bool RED>
 __device__ __forceinline__ void fused_step_warp_item(const StepArgs<T>& a, int item,
                                                 unsigned char* smem_raw) {
 
@@ -203,7 +218,7 @@ __device__ __forceinline__ void fused_step_warp_item(const StepArgs<T>& a, int i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
+            if (line) warp_wake<RED>(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }
@@ -267,7 +282,7 @@ fused_step_warp(const StepArgs<T> a) {
   const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int witem = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); witem < nitems;
        witem += nwarps)
-    fused_step_warp_item<T, TY>(a, a.work ? a.work[witem] : witem, smem_raw);
+    fused_step_warp_item<T, TY, true>(a, a.work ? a.work[witem] : witem, smem_raw);
 }
 
 // Batched form: one launch advances every active member of a batch by one
@@ -284,7 +299,7 @@ fused_step_warp_batch(const BatchMember<T>* __restrict__ members,
     const int2 e = work[witem];
     const BatchMember<T>& mb = members[e.x];
     if (!mb.active) continue;
-    fused_step_warp_item<T, TY>(mb.a, e.y, smem_raw);
+    fused_step_warp_item<T, TY, false>(mb.a, e.y, smem_raw);
   }
 }
 
@@ -461,7 +476,7 @@ __device__ __forceinline__ void fused_step_warp_reg_item(const StepArgs<T>& a, i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
+            if (line) warp_wake<false>(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }
@@ -740,7 +755,7 @@ __device__ __forceinline__ void fused_step_warp_mat_item(const StepArgs<T>& a, i
           if (own_r) {
             oez[id] = ezn;
             ohy[id] = hyn;
-            if (line) add_wake(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
+            if (line) warp_wake<false>(a.b, (a.n + a.b.kshift) - k - a.b.c0, ezn);
           }
           if (r - 1 >= 2 && r - 1 < own_r_end) ohx[id - PX] = hxn_p;
         }
