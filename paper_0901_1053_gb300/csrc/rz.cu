@@ -2380,28 +2380,45 @@ int rz_occupancy(tetm_rz* s) {
   return TETM_OK;
 }
 
+// scratch of at least n ints for the item flags and the plane hulls
+int rz_reserve_flags(tetm_rz* s, int n) {
+  if (n <= s->flags_cap) return TETM_OK;
+  cudaFree(s->flags);
+  s->flags = nullptr;
+  s->flags_cap = 0;
+  cudaError_t e = cudaMalloc(&s->flags, sizeof(int) * (size_t)n);
+  if (e != cudaSuccess) return rz_fail(e);
+  s->flags_cap = n;
+  return TETM_OK;
+}
+
+// Per (tile, chunk) of the windows in use: whether it holds an active entry.
+int rz_flags(tetm_rz* s, int tw, int tiles, int n_chunks, std::vector<int>* fl) {
+  const int nf = tiles * n_chunks;
+  const int rc = rz_reserve_flags(s, nf);
+  if (rc != TETM_OK) return rc;
+  fl->resize((size_t)nf);
+  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, s->L, tiles, tw, s->chunk_z, n_chunks, s->flags);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(fl->data(), s->flags, sizeof(int) * (size_t)nf, cudaMemcpyDeviceToHost, s->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+  return e == cudaSuccess ? TETM_OK : rz_fail(e);
+}
+
+int rz_tile_width(const tetm_rz* s) { return rz_kernel(s) == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile; }
+
 // All of it is made before anything of the solve changes: a rebuild that fails
 // leaves the windows and the item list as they were, fit for each other.
 int rz_rebuild_work(tetm_rz* s) try {
   const RzLayout& L = s->L;
-  const int tw = rz_kernel(s) == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile;
+  const int tw = rz_tile_width(s);
   const int tiles = (L.nr + 1 + tw - 1) / tw, n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
   const int nf = tiles * n_chunks;
-  if (nf > s->flags_cap) {
-    cudaFree(s->flags);
-    s->flags = nullptr;
-    s->flags_cap = 0;
-    cudaError_t e = cudaMalloc(&s->flags, sizeof(int) * (size_t)nf);
-    if (e != cudaSuccess) return rz_fail(e);
-    s->flags_cap = nf;
-  }
-  std::vector<int> fl((size_t)nf);
-  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, L, tiles, tw, s->chunk_z, n_chunks, s->flags);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return rz_fail(e);
-  e = cudaMemcpyAsync(fl.data(), s->flags, sizeof(int) * (size_t)nf, cudaMemcpyDeviceToHost, s->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-  if (e != cudaSuccess) return rz_fail(e);
+  std::vector<int> fl;
+  const int rc = rz_flags(s, tw, tiles, n_chunks, &fl);
+  if (rc != TETM_OK) return rc;
+  cudaError_t e = cudaSuccess;
   std::vector<int> w, first((size_t)n_chunks + 1, 0);
   long long processed = 0;
   for (int q = 0; q < nf; ++q) {
@@ -2476,31 +2493,37 @@ int rz_reshape(tetm_rz* s, int kernel, int chunk_z, bool retile) {
 // us a step on the pair kernel: 512 x 4096, modes 0..4 (130 000 window planes,
 // 1824 warps): 54 with 4 planes, 45 with 8, 41 with 16, 53 with 32, 67 with 48;
 // 93 x 771, mode 0 (1000 window planes): 7.6 with 4, 10.3 with 8, 28.7 with 32.
-int rz_default_chunk(tetm_rz* s) {
-  int rc = rz_rebuild_work(s);
+int rz_default_chunk(tetm_rz* s) try {
+  const int tw = rz_tile_width(s), nz = s->L.nz;
+  const int tiles = (s->L.nr + 1 + tw - 1) / tw, n_chunks = (nz + s->chunk_z - 1) / s->chunk_z;
+  const int least = s->esz == 8 ? 8 : s->mat ? 4 : 2;  // (the one-step sweeps start later)
+  // (one allocation for the flags of every chunk length there can be and the hulls of rz_build_band)
+  int rc = rz_reserve_flags(s, std::max(tiles * ((nz + least - 1) / least), 2 * nz));
   if (rc != TETM_OK) return rc;
-  const long long planes = (long long)s->n_work * s->n_modes * s->chunk_z;
-  const long long least = s->esz == 8 ? 8 : s->mat ? 4 : 2;  // (the one-step sweeps start later)
-  const int cz = (int)std::min(16LL, std::max(least, planes / (4LL * 4 * std::max(1, s->resident)) / 2 * 2));
-  if (cz >= s->L.nz) return TETM_OK;
-  s->chunk_z = cz;
+  std::vector<int> fl;
+  rc = rz_flags(s, tw, tiles, n_chunks, &fl);
+  if (rc != TETM_OK) return rc;
+  const long long planes = (long long)std::count_if(fl.begin(), fl.end(), [](int f) { return f != 0; }) * s->n_modes * s->chunk_z;
+  const int cz = (int)std::min(16LL, std::max((long long)least, planes / (4LL * 4 * std::max(1, s->resident)) / 2 * 2));
+  if (cz < nz) s->chunk_z = cz;
   return rz_rebuild_work(s);
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
 }
 
 // Work items of the float64 band kernels {first plane, planes, first column,
 // columns}: runs of planes with about as many entries as the size of the
 // solve asks for, their columns between the first and last active one.
-int rz_build_band(tetm_rz* s) {
+int rz_build_band(tetm_rz* s) try {
   const RzLayout& L = s->L;
-  int2* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, sizeof(int2) * (size_t)L.nz);
-  if (e != cudaSuccess) return rz_fail(e);
   std::vector<int2> h((size_t)L.nz);
+  const int rc = rz_reserve_flags(s, 2 * L.nz);
+  if (rc != TETM_OK) return rc;
+  int2* d = reinterpret_cast<int2*>(s->flags);
   rz_plane_hulls<<<(L.nz + 7) / 8, 256, 0, s->st>>>(s->mask, L, d);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(int2) * h.size(), cudaMemcpyDeviceToHost, s->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-  cudaFree(d);
   if (e != cudaSuccess) return rz_fail(e);
   long long total = 0;
   for (const int2& v : h) total += v.y - v.x;
@@ -2538,6 +2561,8 @@ int rz_build_band(tetm_rz* s) {
   e = cudaMalloc(&s->band, sizeof(int4) * items.size());
   if (e == cudaSuccess) e = cudaMemcpy(s->band, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
   return e == cudaSuccess ? TETM_OK : rz_fail(e);
+} catch (const std::bad_alloc&) {
+  return TETM_E_NOMEM;
 }
 
 // Per-radian metric of one mode at radial index i (unscaled M^-1; zero where
