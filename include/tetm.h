@@ -83,11 +83,11 @@ typedef struct tetm_info {
   int64_t step;            /* n of the current state y^n                     */
   int64_t device_bytes;    /* device memory held by the solve                */
   int64_t active_cells;    /* cells that carry at least one non-PEC object   */
-  int64_t processed_cells; /* cells the fused kernel reads and writes a step */
+  int64_t processed_cells; /* cells the items of a step own, on the step's kernels */
   int32_t kernel;          /* TETM_KERNEL_*                                  */
   int32_t precision;       /* TETM_FP64 / TETM_FP32                          */
-  int32_t tile_x, tile_y, chunk_z; /* fused-kernel block shape               */
-  int32_t work_items;      /* (tile, z-chunk) blocks launched per step       */
+  int32_t tile_x, tile_y, chunk_z; /* work shape (tetm_set_tiling)           */
+  int32_t work_items;      /* items of that shape, which the balances walk   */
   int32_t wake_len;        /* wake samples (0 before tetm_set_bunch)         */
   int32_t uniform_material;/* 1 if every active coefficient of a component is equal */
 } tetm_info;
@@ -254,16 +254,20 @@ int tetm_set_kernel(tetm_solver* s, int32_t kernel);
  * nodes; each gives TETM_E_UNSUPPORTED for the other kind of solve and in
  * float64; the float32 defaults, with chunks of 4 to 64 planes chosen for the
  * geometry so that the items fill the GPU in whole rounds until a chunk is
- * set; in a batch for the member's share of it);
+ * set, anew whenever the shape changes; in a batch for the member's share of
+ * it). On 56 x 28 items may be shorter than a set chunk, down to half of it,
+ * where the whole length would leave the GPU's last round nearly empty;
  * tile_x = 28 the warp-tiled kernel (one warp per item, tile_y in {4, 8,
  * 12, 16, 20, 28}); tile_x = 32 (tile_y in {4, 8, 16}) or
  * 64 (tile_y in {4, 8}) the block-tiled kernel (one material only). A float64
  * solve whose shape was never set steps in two launches, one per half of the
  * step, over bands of rows of every plane (not a z-slab, which runs the
- * warp-tiled kernel; the shape reported, 28 x 20 x 32, is then the one the
- * balances walk), and so does a small float32 one of one material, over runs
- * of planes of 56 x 14 nodes; the fields are the same bits on all of them. Any value
- * 0 keeps the current one. TETM_E_ARG for other values. */
+ * warp-tiled kernel), and so does a small float32 one of one material, over
+ * runs of planes of 56 x 14 nodes; tile_x, tile_y, chunk_z and work_items of
+ * tetm_get_info are then those the balances walk (float64: 28 x 20 x 32), and
+ * processed_cells is what the two launches step. The fields are the same bits
+ * on all of them. Any value 0 keeps the current one, and a call of zeros alone
+ * the library's choice. TETM_E_ARG for other values. */
 int tetm_set_tiling(tetm_solver* s, int32_t tile_x, int32_t tile_y, int32_t chunk_z);
 
 /* Time-stepping scheme (TETM_SCHEME_*), before the first step. Yee's scheme

@@ -81,7 +81,10 @@ typedef struct tetm_rz_info {
   int32_t work_items;       /* (mode, radial tile, z chunk) items per step      */
   int32_t wake_len;         /* samples of each mode's wake, 0 without a bunch  */
   int32_t resident_warps;   /* step-kernel warps resident on the device at once */
-  int32_t kernel;           /* TETM_RZ_KERNEL_*                                 */
+  int32_t kernel;           /* TETM_RZ_KERNEL_* (until one is set: the library's choice;
+                               float64 then steps in two launches over runs of planes,
+                               which processed_cells counts, and takes this one, chunk_z
+                               and work_items for the scattered-field form)     */
 } tetm_rz_info;
 
 typedef struct tetm_rz tetm_rz;

@@ -567,6 +567,8 @@ int build_band(tetm_solver* s) try {
   std::vector<int4> items;
   band_list(s->L, rows, h, &items, &s->band_smem);
   s->n_band = (int)items.size();
+  s->band_cells = 0;
+  for (const int4& v : items) s->band_cells += (long long)(v.w & 0xFFFF) * (v.w >> 16);
   if (items.empty()) return TETM_OK;
   const int rc = dalloc(s, (void**)&s->band, sizeof(int4) * items.size());
   if (rc != TETM_OK) return rc;
@@ -767,9 +769,7 @@ int do_steps(tetm_solver* s, int n) {
     } else if (s->kernel == TETM_KERNEL_FUSED) {
       StepArgs<T> a = step_args<T>(s, true);
       if (s->n_work > 0) {
-        bool band = false, half = false;
-        if constexpr (sizeof(T) == 8) band = s->band && !s->own_shape;
-        if constexpr (sizeof(T) == 4) half = s->half && !s->own_shape;
+        const bool band = sizeof(T) == 8 && s->bands(), half = sizeof(T) == 4 && s->halves();
         if (band) {
           if constexpr (sizeof(T) == 8) CK(launch_band_step(a, s->band, s->n_band, s->band_smem, s->stream));
           a.b.obs_on = 0;  // the transverse wake is in
@@ -1534,7 +1534,10 @@ int tetm_get_info(tetm_solver* s, tetm_info* info) {
   info->step = s->step;
   info->device_bytes = s->device_bytes;
   info->active_cells = s->active_cells;
-  info->processed_cells = (long long)s->n_work * s->tile_x * slab_rows(s->tile_x, s->tile_y) * s->item_z;
+  const bool fused = s->scheme == TETM_SCHEME_TETM && s->kernel == TETM_KERNEL_FUSED && !s->in_batch;
+  info->processed_cells = fused && s->bands()    ? s->band_cells
+                          : fused && s->halves() ? (long long)s->n_half * kHalfX * kHalfY * s->half_run
+                                                 : (long long)s->n_work * s->tile_x * slab_rows(s->tile_x, s->tile_y) * s->item_z;
   info->kernel = s->kernel;
   info->precision = s->g.precision;
   info->tile_x = s->tile_x;

@@ -2044,6 +2044,7 @@ struct tetm_rz {
   bool own_shape = false;        // the caller chose a kernel or a chunk length
   int4* band = nullptr;          // float64: work items of the band kernels
   int n_band = 0, band_smem = 0;
+  long long band_entries = 0;    // of one mode, which they own
   bool te_zero = true;           // nothing has set e_phi, h_r, h_z of mode 0
   bool work_dirty = true;
   long long processed = 0;
@@ -2114,6 +2115,9 @@ constexpr int kSourcePlanes = 2;  // planes per source work item
 int rz_kernel(const tetm_rz* s) {
   return !s->own_shape && s->esz == 4 && !s->mat ? TETM_RZ_KERNEL_BULK2 : s->kernel;
 }
+
+// a float64 solve steps on the band kernels (the source windows are the other kernels')
+bool rz_bands(const tetm_rz* s) { return s->band && !s->own_shape && !s->scattered; }
 
 // Sources of the scattered-field form for steps s->step .. s->step + n_steps - 1.
 template <typename T>
@@ -2220,7 +2224,7 @@ int rz_launch_steps(tetm_rz* s, long long n) {
   a.changes = s->changes;
   a.change_words = s->change_words;
   a.sched = s->err + 2;
-  const bool band = s->band && !s->own_shape && !s->scattered;  // (the source windows are the other kernels')
+  const bool band = rz_bands(s);
   const int items = s->n_work * s->n_modes;
   const int blocks = std::max(1, std::min(s->resident, (items + 3) / 4));
   // launches one step kernel over the plain items (SC = false) or over the
@@ -2556,6 +2560,8 @@ int rz_build_band(tetm_rz* s) try {
     k += n;
   }
   s->n_band = (int)items.size();
+  s->band_entries = 0;
+  for (const int4& v : items) s->band_entries += (long long)v.y * v.w;
   s->band_smem = top * s->esz;
   if (items.empty()) return TETM_OK;
   e = cudaMalloc(&s->band, sizeof(int4) * items.size());
@@ -3269,13 +3275,13 @@ int tetm_rz_get_info(tetm_rz* s, tetm_rz_info* info) {
   if (!s || !info) return TETM_E_ARG;
   info->step = s->step;
   info->device_bytes = s->device_bytes;
-  info->processed_cells = s->processed;
+  info->processed_cells = rz_bands(s) ? s->band_entries * s->n_modes : s->processed;
   info->n_modes = s->n_modes;
   info->chunk_z = s->chunk_z;
   info->work_items = s->n_work * s->n_modes;
   info->wake_len = s->bunch ? s->nw : 0;
   info->resident_warps = 4 * s->resident;
-  info->kernel = s->kernel;
+  info->kernel = rz_kernel(s);
   return TETM_OK;
 }
 

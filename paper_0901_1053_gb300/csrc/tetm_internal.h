@@ -288,9 +288,13 @@ struct tetm_solver {
   std::vector<uint8_t> act;    // per tile and plane (tile-major): the tile owns an active cell there
   int4* band;                  // float64: work items of the band kernels (the default work shape)
   int n_band, band_smem;
+  long long band_cells;        // nodes they own
   int* half;                   // float32, small grids: work items of the half-step kernels (tile + tiles * run)
   int n_half, half_run;        // planes per item
   std::vector<int> work_host;  // host copy of the work list
+  // which step a fused TE/TM solve takes: bands or half-steps until a shape is set
+  bool bands() const { return band && !own_shape; }
+  bool halves() const { return half && !own_shape; }
   // the slab kernel's shape: planes per item by choose_chunk unless set
   bool auto_chunk() const { return esz == 4 && tetm::slab_shape_ok(tile_x, tile_y, !uniform); }
   bool in_batch;               // stepped by a tetm_batch
