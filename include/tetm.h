@@ -420,7 +420,8 @@ int tetm_batch_step(tetm_batch* b, int32_t nsteps);
 /* Wait for the batch's stream (synchronizes). */
 int tetm_batch_sync(tetm_batch* b);
 
-/* Members, members below their limit, and (member, item) work entries. */
+/* Members, members below their limit, and the (member, item) work entries of
+ * those. */
 int tetm_batch_info(tetm_batch* b, int32_t* n_members, int32_t* n_active, int32_t* work_items);
 
 /* Release the batch (synchronizes); members become independent again. */

@@ -49,7 +49,6 @@ struct tetm_batch {
   void* d_members;                 // BatchMember<T>[capacity]
   int* d_wbuf;                     // kHead ints (entry count first), then int2 entries
   int wcap;                        // entries d_wbuf holds
-  int n_work;                      // entries of the list last uploaded
   bool work_dirty;                 // membership changed since
   int nz_max;                      // transverse-wake grid bound of the launches (0: no member gathers)
   cudaStream_t stream;
@@ -152,7 +151,6 @@ int upload_work(tetm_batch* b) {
   h[0] = n;
   const int rc = stage_copy(b, b->d_wbuf, h.data(), sizeof(int) * h.size());
   if (rc != TETM_OK) return rc;
-  b->n_work = n;
   b->work_dirty = false;
   return TETM_OK;
 }
@@ -512,15 +510,18 @@ int tetm_batch_sync(tetm_batch* b) {
 int tetm_batch_info(tetm_batch* b, int32_t* n_members, int32_t* n_active, int32_t* work_items) {
   if (!b) return TETM_E_ARG;
   int mem = 0, act = 0;
+  long long items = 0;  // what the list holds at the next step: retired members' items leave it on the device
   for (int i = 0; i < b->capacity; ++i) {
     tetm_solver* s = b->slot[(size_t)i];
     if (!s) continue;
     ++mem;
-    if (s->step < b->limit[(size_t)i]) ++act;
+    if (s->step >= b->limit[(size_t)i]) continue;
+    ++act;
+    items += (long long)b->items[(size_t)i].size();
   }
   if (n_members) *n_members = mem;
   if (n_active) *n_active = act;
-  if (work_items) *work_items = b->n_work;
+  if (work_items) *work_items = (int32_t)items;
   return TETM_OK;
 }
 

@@ -101,6 +101,34 @@ def test_a_batch_member_reports_its_items(tetm):
     s.close()
 
 
+def test_batch_work_items_are_those_still_stepped(tetm):
+    """(member, item) entries of the members below their limit, before and after members retire, join and leave."""
+    dims = [(64, 64, 130), (57, 13, 5), (113, 25, 67)]
+    for tile in ((56, 28), (28, 20)):
+        b = tetm.Batch.slots(3, "fp32", tile, graph_steps=2)
+        assert b.info()["work_items"] == 0
+        per = {}
+        members = []
+        for d, limit in zip(dims, (2, 5, 9)):
+            s = cartesian(tetm, d, "fp32")
+            before = b.info()["work_items"]
+            b.add(s, limit)
+            per[limit] = b.info()["work_items"] - before
+            members.append(s)
+        assert all(per.values())
+        for step in range(1, 11):
+            b.step(1)
+            assert b.info()["work_items"] == sum(n for limit, n in per.items() if step < limit)
+        extra = cartesian(tetm, dims[0], "fp32")
+        b.remove(members[0])
+        b.add(extra, 3)
+        assert b.info()["work_items"] == per[2]
+        b.remove(extra)
+        assert b.info()["work_items"] == 0
+        b.sync()
+        b.close()
+
+
 def test_rz_reports_the_kernel_that_steps(tetm):
     pec = wl.cavity_chain_rz(57, 70, 0, 1).pec
     cells = int((pec == 0).sum())
