@@ -467,12 +467,21 @@ def run_tetm(args):
                 "achieved_on_processed_cells": FLOPS_PER_CELL_3D * proc / (kern_ms * 1e-3) / 1e12,
                 "hbm_gbs": gbs, "bytes_per_cell": bytes_per_cell}
     kname = {28: "fused_step_warp", 56: "fused_step_slab"}.get(info["tile_x"], "fused_step")
+    # a solve whose shape was not set and whose step is not that of the shape reported: two launches a step
+    shape_cells = (info["work_items"] * info["tile_x"] * (12 if info["tile_x"] == 56 else info["tile_y"])
+                   * info["chunk_z"])
+    two_launches = (args.kernel == "fused" and not any(args.tiling_used or ())
+                    and info["processed_cells"] != shape_cells)
+    if two_launches:
+        kname = "band_step" if w.precision == "fp64" else "half_step"
     if args.kernel == "twostep":
         kname = "fused_step2"
-    if args.eps is not None:
+    if args.eps is not None and not two_launches:
         kname = "fused_step_slab_mat" if info["tile_x"] == 56 else "fused_step_warp_mat"
     prof_name = "%s_%s_%s.md" % (kname, w.precision, w.name)
-    sources = ("kernels_slab.cu",) if kname.startswith("fused_step_slab") else ("kernels_step.cu", "kernels_warp.cu")
+    sources = {"fused_step_slab": ("kernels_slab.cu",), "fused_step_slab_mat": ("kernels_slab.cu",),
+               "band_step": ("kernels_band.cu",), "half_step": ("kernels_half.cu",)}.get(
+                   kname, ("kernels_step.cu", "kernels_warp.cu"))
     traffic = (profiled_traffic(prof_name, sources, (info["tile_x"], info["tile_y"], info["chunk_z"]))
                if args.kernel != "reference" else None)
     wake = s.wake()[0]
@@ -563,8 +572,9 @@ def run_tetm(args):
         # per balance: the bunch charge, the one fused pass and its second
         # reduction pass (one material); energy and charge passes separately
         # (material arrays)
-        "gpu_launches": ((10 * K if args.kernel == "reference" else (K // 2 if args.kernel == "twostep" else K))
-                         + (3 if args.eps is None else 6) * n_bal),
+        "gpu_launches": (10 * K if args.kernel == "reference" else K // 2 if args.kernel == "twostep"
+                         else 2 * K if two_launches else K)
+                        + (3 if args.eps is None else 6) * n_bal,
         "clocks": clk,
         "balances": {"records": int(hist.shape[0]), "in_timed_region": n_bal,
                      "ms_per_balance": bal_ms,
@@ -782,8 +792,12 @@ def run_rz_mode(args):
         kern, chunk = tune_rz(w)
         kern = args.rz_kernel or kern
         chunk = args.rz_chunk or chunk
+    if kern == "default" and args.rz_chunk:
+        kern = "async"
+    bands = kern == "default" and args.rz_start != "scattered"   # two launches a step
     s.set_kernel(kern)
-    s.set_tiling(chunk)
+    if chunk:
+        s.set_tiling(chunk)
     info = s.info()
     s.step(args.warmup)
     s.sync()
@@ -816,7 +830,8 @@ def run_rz_mode(args):
     bytes_per_cell = 12 * esz + 1
     proc = info["processed_cells"]
     kname = {"async": "rz_step_async_kernel", "bulk": "rz_step_bulk_kernel",
-             "bulk2": "rz_step_bulk2_kernel"}.get(kern, "rz_step_kernel")
+             "bulk2": "rz_step_bulk2_kernel", "default": "rz_band" if bands else "rz_step_async_kernel"}.get(
+                 kern, "rz_step_kernel")
     launch_ms = kern_ms * stride           # one launch reads y^n and writes y^{n+stride}
     if w.precision == "fp32":
         achieved = bytes_per_cell * proc / (launch_ms * 1e-3) / 1e9
@@ -844,7 +859,8 @@ def run_rz_mode(args):
         s2 = tetm.RzSolver(w.nr, w.nz, w.m_lo, w.m_hi, w.dr, w.dz, w.cdt, w.precision, pec=pinned)
         rz_start(s2, w, args.rz_start)
         s2.set_kernel(kern)
-        s2.set_tiling(chunk)
+        if chunk:
+            s2.set_tiling(chunk)
         s2.step(steps_e2e)
         wakes = [s2.wake(m)[0] for m in range(w.m_lo, w.m_hi + 1)]
         t1 = time.perf_counter()
@@ -903,7 +919,7 @@ def run_rz_mode(args):
         "e2e": e2e,
         # per pass: the plain step kernel, plus in the scattered form the same
         # kernel over the items meeting the source window, and the sources
-        "gpu_launches": R * (2 if args.rz_start == "scattered" else 1)
+        "gpu_launches": R * (2 if bands or args.rz_start == "scattered" else 1)
                         + rz_source_launches(args.rz_start, args.warmup, K, stride),
         "clocks": clk,
     }

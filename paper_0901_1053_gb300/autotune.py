@@ -1,10 +1,11 @@
 """Work-shape autotuner for the fused step kernels.
 
 For a grid and geometry it times candidate (tile_x, tile_y, chunk_z) shapes
-on a scratch solve with the same geometry (the cost of a step does not depend
-on the bunch or on the field values), keeps the fastest and caches it in a
-JSON file keyed by GPU name, precision, grid size and a digest of the PEC
-mask. Tuning runs solves through the C ABI only; nothing here computes fields.
+and the library's own choice on a scratch solve with the same geometry (the
+cost of a step does not depend on the bunch or on the field values), keeps the
+fastest and caches it in a JSON file keyed by GPU name, precision, grid size
+and a digest of the PEC mask. Tuning runs solves through the C ABI only;
+nothing here computes fields.
 """
 from __future__ import annotations
 
@@ -17,6 +18,11 @@ from typing import Dict, List, Optional, Sequence, Tuple
 import numpy as np
 
 Shape = Tuple[int, int, int]
+
+# The library's choice, as set_tiling takes it on a solve whose shape was never
+# set: float64 and small float32 solves then step in two launches, which no
+# shape names (11 to 73 and 2 times faster than the best of the shapes).
+DEFAULT: Shape = (0, 0, 0)
 
 CANDIDATES_FP32: List[Shape] = [(56, 28, 32), (56, 28, 16), (56, 28, 64), (56, 12, 32), (56, 12, 16),
                                 (28, 20, 32), (28, 20, 16), (28, 12, 32), (28, 12, 16),
@@ -52,6 +58,7 @@ class Autotuner:
         self.steps = steps
         self.warmup = warmup
         self.repeats = repeats
+        self.default_seconds: Optional[float] = None   # a step on the library's choice (measure)
         self.cache: Dict[str, list] = {}
         if os.path.exists(self.path):
             try:
@@ -76,29 +83,34 @@ class Autotuner:
 
     def measure(self, w, precision: str, shapes: Sequence[Shape], eps_r=None) -> Dict[Shape, float]:
         """Seconds per step of each shape on a scratch solve of w's geometry
-        (and material array eps_r, which selects the coefficient-array kernels)."""
+        (and material array eps_r, which selects the coefficient-array kernels);
+        those of the library's choice, before any shape is set, in default_seconds."""
         from . import tetm
         s = tetm.Solver(w.nx, w.ny, w.nz, w.dx, w.dy, w.dz, w.cdt, precision, eps_r=eps_r, pec=w.pec)
         out = {}
         try:
+            self.default_seconds = self._time(s)
             for shape in shapes:
                 try:
                     s.set_tiling(*shape)
                 except tetm.TetmError:
                     continue
-                s.step(self.warmup)
-                s.sync()
-                best = None
-                for _ in range(self.repeats):  # the fastest of a few runs: less noise from the host
-                    t0 = time.perf_counter()
-                    s.step(self.steps)
-                    s.sync()
-                    dt = (time.perf_counter() - t0) / self.steps
-                    best = dt if best is None else min(best, dt)
-                out[tuple(shape)] = best
+                out[tuple(shape)] = self._time(s)
         finally:
             s.close()
         return out
+
+    def _time(self, s) -> float:
+        s.step(self.warmup)
+        s.sync()
+        best = None
+        for _ in range(self.repeats):  # the fastest of a few runs: less noise from the host
+            t0 = time.perf_counter()
+            s.step(self.steps)
+            s.sync()
+            dt = (time.perf_counter() - t0) / self.steps
+            best = dt if best is None else min(best, dt)
+        return best
 
     def wave_fitted(self, w, precision: str, tile_ys=(12, 20, 28), max_extra: int = 6, eps_r=None):
         """Shapes (28, ty, cz) whose work-item count fills whole waves of the
@@ -153,7 +165,10 @@ class Autotuner:
         """materials: the solve has eps/mu arrays (per-entry coefficients run on
         the warp-tiled kernel, tile_x = 28, and the float32 slab kernel, 56 x 12);
         batch: the shape is for a batch of solves (batched launches run the
-        warp-tiled kernel, tile_x = 28, and in float32 the slab kernel)."""
+        warp-tiled kernel, tile_x = 28, and in float32 the slab kernel).
+        (0, 0, 0) where the library's choice is the fastest: set_tiling takes it
+        on a new solve. A batch steps on a shape, and candidates that are given
+        are the only ones."""
         precision = precision or w.precision
         materials = materials or eps_r is not None
         k = self.key(w, precision) + ("|materials56x12" if materials else "") + ("|batch" if batch else "")
@@ -170,7 +185,10 @@ class Autotuner:
             cands = [c for c in cands if (c[0], c[1]) != (56, 12)]
         if batch:
             cands = [c for c in cands if c[0] == 28 or (precision == "fp32" and (c[0], c[1]) == (56, 28))]
+        self.default_seconds = None
         times = self.measure(w, precision, cands, eps_r=eps_r)
+        if self.default_seconds is not None and candidates is None and not batch:
+            times = {**times, DEFAULT: self.default_seconds}
         best = min(times, key=times.get)
         self.cache[k] = list(best)
         self._save()
@@ -184,25 +202,34 @@ class Autotuner:
 def tune_rz(w, precision: Optional[str] = None, steps: int = 8, warmup: int = 3,
             extra_chunks: Sequence[int] = (16, 24, 32, 64, 128)):
     """(kernel, chunk_z) with the shortest step on a scratch solve of w's
-    geometry: each step kernel with its wave-fitted chunk and a few fixed
-    ones (the two-steps-per-pass kernel timed over pairs of steps). Returns
-    ("bulk2" | "bulk" | "register" | "async", chunk_z)."""
+    geometry: each step kernel with its wave-fitted chunk, a few fixed ones and
+    the library's own (the two-steps-per-pass kernel timed over pairs of steps).
+    Returns ("bulk2" | "bulk" | "register" | "async", chunk_z), or ("default", 0)
+    where the library's choice for float64, two launches that no kernel names,
+    is the fastest (in float32 its choice is "bulk2" with a chunk of its own)."""
     from . import tetm
     precision = precision or w.precision
     s = tetm.RzSolver(w.nr, w.nz, w.m_lo, w.m_hi, w.dr, w.dz, w.cdt, precision, pec=w.pec)
+
+    def seconds():
+        s.step(2 * warmup)
+        s.sync()
+        t0 = time.perf_counter()
+        s.step(2 * steps)
+        s.sync()
+        return (time.perf_counter() - t0) / (2 * steps)
+
     best = None
     try:
+        own = max(4, s.info()["chunk_z"])
+        if precision == "fp64":
+            best = (seconds(), "default", 0)
         for kern in ("bulk2", "bulk", "register", "async"):
             s.set_kernel(kern)
-            chunks = [s.wave_fitted_chunk()] + [c for c in extra_chunks]
+            chunks = [s.wave_fitted_chunk(), own] + [c for c in extra_chunks]
             for c in dict.fromkeys(chunks):
                 s.set_tiling(c)
-                s.step(2 * warmup)
-                s.sync()
-                t0 = time.perf_counter()
-                s.step(2 * steps)
-                s.sync()
-                dt = (time.perf_counter() - t0) / (2 * steps)
+                dt = seconds()
                 if best is None or dt < best[0]:
                     best = (dt, kern, c)
     finally:

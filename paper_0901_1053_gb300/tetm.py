@@ -547,6 +547,7 @@ class RzSolver:
         self.m_lo, self.m_hi = int(m_lo), int(m_hi)
         self.shape = (self.nz + 1, self.nr + 1)
         self.precision = precision
+        self._shape_set = False
         cell = (self.nz, self.nr)
         arrs = []
         for a, dt in ((eps_r, np.float64), (mu_r, np.float64), (pec, np.uint8)):
@@ -585,12 +586,20 @@ class RzSolver:
 
     def set_tiling(self, chunk_z):
         _check(lib.tetm_rz_set_tiling(self.h, int(chunk_z)), "tetm_rz_set_tiling")
+        self._shape_set = True
 
     def set_kernel(self, kernel):
+        """A step kernel, or "default": the library's choice, on a solve whose
+        kernel and chunk were never set."""
+        if kernel == "default":
+            if self._shape_set:
+                raise ValueError("the kernel or the chunk of this solve was set")
+            return
         k = {"async": TETM_RZ_KERNEL_ASYNC, "register": TETM_RZ_KERNEL_REGISTER,
              "bulk": TETM_RZ_KERNEL_BULK, "bulk2": TETM_RZ_KERNEL_BULK2}[kernel] \
             if isinstance(kernel, str) else int(kernel)
         _check(lib.tetm_rz_set_kernel(self.h, k), "tetm_rz_set_kernel")
+        self._shape_set = True
 
     def set_stream(self, stream):
         _check(lib.tetm_rz_set_stream(self.h, ctypes.c_void_p(int(stream) if stream else 0)),
@@ -694,7 +703,8 @@ class RzSolver:
     def wave_fitted_chunk(self, lo=24, hi=256):
         """Planes per work item whose item count fills whole waves of the
         resident warps best (ties go to the longer chunk); leaves that tiling
-        set."""
+        set (a float64 solve then steps on a named kernel, not on the library's
+        two launches)."""
         best = None
         for c in range(lo, hi + 1, 4):
             self.set_tiling(c)
