@@ -3,12 +3,14 @@
 For a grid and geometry it times candidate (tile_x, tile_y, chunk_z) shapes
 and the library's own choice on a scratch solve with the same geometry (the
 cost of a step does not depend on the bunch or on the field values), keeps the
-fastest and caches it in a JSON file keyed by GPU name, precision, grid size
-and a digest of the PEC mask. Tuning runs solves through the C ABI only;
+fastest and caches it in a JSON file keyed by GPU name, precision, grid size, a
+digest of the PEC mask and one of the library's sources (a shape tuned for
+other kernels is not an answer). Tuning runs solves through the C ABI only;
 nothing here computes fields.
 """
 from __future__ import annotations
 
+import glob
 import hashlib
 import json
 import os
@@ -52,6 +54,17 @@ def geometry_digest(pec) -> str:
     return hashlib.sha1(memoryview(pec).tobytes()).hexdigest()[:16]
 
 
+def library_digest() -> str:
+    """Of the kernels a tuned shape is for: their sources, or the built library where those are not there."""
+    from .build import CSRC, library_path
+    files = sorted(glob.glob(os.path.join(CSRC, "*"))) or [library_path()]
+    h = hashlib.sha1()
+    for p in files:
+        with open(p, "rb") as f:
+            h.update(os.path.basename(p).encode() + b"\0" + f.read())
+    return h.hexdigest()[:16]
+
+
 class Autotuner:
     def __init__(self, cache_path: Optional[str] = None, steps: int = 20, warmup: int = 3, repeats: int = 2):
         self.path = cache_path or default_cache_path()
@@ -69,7 +82,7 @@ class Autotuner:
 
     def key(self, w, precision: str) -> str:
         return "|".join([_gpu_name(), precision, "%dx%dx%d" % (w.nx, w.ny, w.nz),
-                         geometry_digest(w.pec)])
+                         geometry_digest(w.pec), library_digest()])
 
     def _save(self):
         try:

@@ -1,11 +1,11 @@
-"""The autotuners' answer where the library's own choice is the fastest step, which no shape or kernel name names.
-Host logic only: timings are stand-ins."""
+"""The autotuners' answer where the library's own choice is the fastest step, which no shape or kernel name names, and
+a cache that outlived the kernels it was filled for. Host logic only: timings are stand-ins."""
 import types
 
 import numpy as np
 import pytest
 
-from paper_0901_1053_gb300 import autotune, tetm
+from paper_0901_1053_gb300 import autotune, build, tetm
 
 
 def workload(precision="fp32"):
@@ -73,6 +73,19 @@ def test_measure_times_the_librarys_choice_before_any_shape(monkeypatch):
     out = t.measure(w, "fp64", [(28, 20, 32), (32, 8, 64)])
     assert list(out) == [(28, 20, 32)] and t.default_seconds > 0
     assert calls == [2, 7, (28, 20, 32), 2, 7, "close"]
+
+
+def test_a_cache_filled_for_other_kernels_is_not_used(tmp_path, monkeypatch):
+    src = tmp_path / "csrc"
+    src.mkdir()
+    (src / "k.cu").write_text("// a kernel\n")
+    monkeypatch.setattr(build, "CSRC", str(src))
+    t = Timed(tmp_path / "c.json", 2.0)
+    first = t.tune(workload())
+    assert t.tune(workload()) == first and t.calls == 1
+    (src / "k.cu").write_text("// the kernel, changed\n")
+    u = Timed(tmp_path / "c.json", 0.5)
+    assert u.tune(workload()) == (0, 0, 0) and u.calls == 1
 
 
 class Rz:
