@@ -38,6 +38,7 @@
 #include <new>
 #include <vector>
 
+#include "quads.cuh"
 #include "tetm_internal.h"
 #include "tetm_rz.h"
 #include <nvtx3/nvToolsExt.h>
@@ -47,6 +48,7 @@ namespace {
 using tetm::kC;
 using tetm::kEps0;
 using tetm::kMu0;
+using tetm::f2, tetm::pk, tetm::lo, tetm::hi;
 
 constexpr int kER = TETM_RZ_ER, kEP = TETM_RZ_EPHI, kEZ = TETM_RZ_EZ;
 constexpr int kHR = TETM_RZ_HR, kHP = TETM_RZ_HPHI, kHZ = TETM_RZ_HZ;
@@ -956,22 +958,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) rz_step_bulk2_ker
 // form 56 -> 48. What is left is latency: twelve warps an SM, a chain of about
 // 18 dependent operations and four shuffles per plane and step. Compiled for
 // four blocks an SM it spills: 49 us.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 pk(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float lo(f2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return a;
-}
-__device__ __forceinline__ float hi(f2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return b;
-}
 __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
   f2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -2520,12 +2506,16 @@ int rz_default_chunk(tetm_rz* s) try {
 // solve asks for, their columns between the first and last active one.
 int rz_build_band(tetm_rz* s) try {
   const RzLayout& L = s->L;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return rz_fail(e);
   std::vector<int2> h((size_t)L.nz);
   const int rc = rz_reserve_flags(s, 2 * L.nz);
   if (rc != TETM_OK) return rc;
   int2* d = reinterpret_cast<int2*>(s->flags);
   rz_plane_hulls<<<(L.nz + 7) / 8, 256, 0, s->st>>>(s->mask, L, d);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(int2) * h.size(), cudaMemcpyDeviceToHost, s->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   if (e != cudaSuccess) return rz_fail(e);
@@ -2534,7 +2524,7 @@ int rz_build_band(tetm_rz* s) try {
   // about six items an SM, of 128 to 512 entries: 256 x 2048 with modes 0, 1
   // takes 46.9 us a step with runs of 128 entries, 43.4 with 256, 42.8 with
   // 512 and 57.3 with 1024 (0.64 M active entries)
-  const long long target = std::min(512LL, std::max(128LL, total * s->n_modes / (152 * 6)));
+  const long long target = std::min(512LL, std::max(128LL, total * s->n_modes / (6LL * sms)));
   std::vector<int4> items;
   int top = 0;
   for (int k = 0; k < L.nz;) {
