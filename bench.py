@@ -482,7 +482,11 @@ def run_tetm(args):
     sources = {"fused_step_slab": ("kernels_slab.cu",), "fused_step_slab_mat": ("kernels_slab.cu",),
                "band_step": ("kernels_band.cu",), "half_step": ("kernels_half.cu",)}.get(
                    kname, ("kernels_step.cu", "kernels_warp.cu"))
-    traffic = (profiled_traffic(prof_name, sources, (info["tile_x"], info["tile_y"], info["chunk_z"]))
+    # planes per item as stepped (a set chunk of 56 x 28 may be shortened)
+    planes = info["chunk_z"]
+    if kname.startswith("fused_step_slab") and info["work_items"]:
+        planes = info["processed_cells"] // (info["work_items"] * info["tile_x"] * 12)
+    traffic = (profiled_traffic(prof_name, sources, (info["tile_x"], info["tile_y"], planes))
                if args.kernel != "reference" else None)
     wake = s.wake()[0]
     hist = s.balance_history()

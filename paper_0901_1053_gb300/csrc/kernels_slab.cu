@@ -9,10 +9,13 @@
 // z-state of its quad in registers (old e_x, e_y, new h_x, h_y of the planes
 // below): no per-row state in shared memory.
 //
-// What bounds it: the shared-memory and load/store pipe together with the
-// latency of the next plane's loads, not DRAM. With one material on 256 x 256
-// x 2048 a step takes 395 us, of which the arithmetic and barriers alone take
-// 209 us, and all inputs from L2 instead of DRAM 373 us. Tried on the way (us
+// What bounds it: latency behind the block barriers at 16 warps per SM. No pipe
+// is full: on 256 x 256 x 512 L1/TEX is at 58% (its shared-memory and
+// load/store data pipe 51), DRAM 55, SM 46, and of a warp's 7.4 cycles per
+// issued instruction 1.9 are a barrier, 1.0 global loads, 0.9 shared memory, 0.5
+// the arithmetic pipes. With one material on 256 x 256 x 2048 a step takes 395
+// us, of which the arithmetic and barriers alone take 209 us, and all inputs
+// from L2 instead of DRAM 373 us. Tried on the way (us
 // per step on 256 x 256 x 1024 / 2048 and on a 16-solve batch's longest
 // solve): one CTA of 512 threads on 64 x 32 boxes in scalar arithmetic 225 /
 // 402 / 534; the same with packed pairs of float32 (half the issue slots for
@@ -20,8 +23,8 @@
 // 395 / 476 and 32.8 instead of 54.7 on 48 x 48 x 192, where a grid of few
 // tiles makes 2.3 times the items. The rows loaded in vain (4 of 16 instead of
 // 4 of 32) cost less than the waits of a lone CTA. A ring for all six inputs
-// instead of register loads, and tensor-map copies into it, were slower (the
-// ring's reads go through the pipe that is full), and so were later loads of
+// instead of register loads, and tensor-map copies into it, were slower (more
+// shared-memory reads between the same barriers), and so were later loads of
 // e_x, e_y (238 us), a sweep unrolled by three planes (264 us: code size) and
 // one that gathers the transverse wake itself (1.3 us more, the launch 1.5 less
 // only on small grids). With coefficient arrays packed pairs save nothing (192 x
@@ -97,7 +100,7 @@ struct SlabSmemU {
 };
 // Material arrays: two-plane rings of e_z and h_z with the six per-entry
 // coefficient arrays (alpha M^-1, 2 alpha M^-1 for e_z and h_z), and the four
-// exchange buffers of the skewed sweep (hx~, ez', ex~, hz'), 160 KB, in one
+// exchange buffers of the skewed sweep (hx~, ez', ex~, hz'), 82 KB, in one
 // array with a spare row at the end (reads past a buffer's edge stay inside).
 struct SlabSmemM {
   static constexpr int kP = kSY * kSX;
@@ -149,9 +152,9 @@ __device__ __forceinline__ void sts4(float* p, const Q4& a) {
 // updates of every plane of the chunk, plane by plane: four block barriers
 // per plane). SHARED: a lies in shared memory (batches) instead of the
 // parameter space. There each array's address is its set's pointer, kept in
-// registers, plus a multiple of cstep: read from shared memory the twelve
-// pointers took a slot each of the pipe that bounds the sweep in every plane
-// (batch of 16 solves: 558 us per step of the longest, so 476). From the
+// registers, plus a multiple of cstep: the twelve pointers were a shared-memory
+// read each in every plane, ahead of the access that needs it (batch of 16
+// solves: 558 us per step of the longest, so 476). From the
 // parameter space the twelve pointers are free, and one running pointer per
 // set was measured 1.7 times slower.
 //

@@ -2483,6 +2483,13 @@ int rz_reshape(tetm_rz* s, int kernel, int chunk_z, bool retile) {
 // us a step on the pair kernel: 512 x 4096, modes 0..4 (130 000 window planes,
 // 1824 warps): 54 with 4 planes, 45 with 8, 41 with 16, 53 with 32, 67 with 48;
 // 93 x 771, mode 0 (1000 window planes): 7.6 with 4, 10.3 with 8, 28.7 with 32.
+// The one-step sweeps gain as well, us a step with 32 planes | the choice: with
+// material arrays 93 x 771 float32 33.5 | 8.5, float64 96 | 7.1, 256 x 2048 modes
+// 0, 1 36.6 | 14.6 and 112 | 46.7, 512 x 4096 modes 0..4 123 | 111 and 537 | 488;
+// the scattered form in float64, 256 x 2048 92 | 67.5, 512 x 4096 513 | 461;
+// single float32 steps (a call of one step), bulk-copy sweep on 56-entry windows
+// against the asynchronous-copy one with 32 planes, 93 x 771 28.6 | 6.3, 512 x
+// 4096 90 | 74.
 int rz_default_chunk(tetm_rz* s) try {
   const int tw = rz_tile_width(s), nz = s->L.nz;
   const int tiles = (s->L.nr + 1 + tw - 1) / tw, n_chunks = (nz + s->chunk_z - 1) / s->chunk_z;
