@@ -1466,14 +1466,18 @@ __global__ void rz_mask_changes(const uint8_t* mask, RzLayout L, int tiles, int 
   if (q >= (long long)tiles * words) return;
   const int tile = (int)(q / words), word = (int)(q % words);
   const long long col = (long long)tile * kTile2 - 4 + L.orr + 2 * lane;  // even, as the pitch
+  // (the 33 rows first, then their comparisons: one memory latency, not 32)
+  unsigned short v[33];
+#pragma unroll
+  for (int b = 0; b < 33; ++b) {
+    const long long row = (long long)word * 32 + b - 1;
+    v[b] = row >= 0 && row < L.rows ? *reinterpret_cast<const unsigned short*>(mask + row * L.pr + col) : 0;
+  }
   unsigned bits = 0;
+#pragma unroll
   for (int b = 0; b < 32; ++b) {
     const long long row = (long long)word * 32 + b;
-    bool d = row == 0;
-    if (row > 0 && row < L.rows)
-      d = *reinterpret_cast<const unsigned short*>(mask + row * L.pr + col) !=
-          *reinterpret_cast<const unsigned short*>(mask + (row - 1) * L.pr + col);
-    if (__any_sync(0xffffffffu, d)) bits |= 1u << b;
+    if (__any_sync(0xffffffffu, row == 0 || (row < L.rows && v[b + 1] != v[b]))) bits |= 1u << b;
   }
   if (lane == 0) out[q] = bits;
 }
@@ -2382,13 +2386,13 @@ int rz_reserve_flags(tetm_rz* s, int n) {
   return TETM_OK;
 }
 
-// Per (tile, chunk) of the windows in use: whether it holds an active entry.
-int rz_flags(tetm_rz* s, int tw, int tiles, int n_chunks, std::vector<int>* fl) {
-  const int nf = tiles * n_chunks;
+// Per (tile, chunk of cz planes) of the windows: whether it holds an active entry.
+int rz_flags(tetm_rz* s, int tw, int tiles, int cz, std::vector<int>* fl) {
+  const int n_chunks = (s->L.nz + cz - 1) / cz, nf = tiles * n_chunks;
   const int rc = rz_reserve_flags(s, nf);
   if (rc != TETM_OK) return rc;
   fl->resize((size_t)nf);
-  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, s->L, tiles, tw, s->chunk_z, n_chunks, s->flags);
+  rz_item_flags<<<(nf + 255) / 256, 256, 0, s->st>>>(s->mask, s->L, tiles, tw, cz, n_chunks, s->flags);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(fl->data(), s->flags, sizeof(int) * (size_t)nf, cudaMemcpyDeviceToHost, s->st);
@@ -2398,16 +2402,12 @@ int rz_flags(tetm_rz* s, int tw, int tiles, int n_chunks, std::vector<int>* fl) 
 
 int rz_tile_width(const tetm_rz* s) { return rz_kernel(s) == TETM_RZ_KERNEL_BULK2 ? kTile2 : kTile; }
 
-// All of it is made before anything of the solve changes: a rebuild that fails
-// leaves the windows and the item list as they were, fit for each other.
-int rz_rebuild_work(tetm_rz* s) try {
+// The item list of windows tw wide and chunks of s->chunk_z planes from their
+// flags. All of it is made before anything of the solve changes: when it fails,
+// the windows and the item list stay as they were, fit for each other.
+int rz_take_list(tetm_rz* s, int tw, int tiles, const std::vector<int>& fl) {
   const RzLayout& L = s->L;
-  const int tw = rz_tile_width(s);
-  const int tiles = (L.nr + 1 + tw - 1) / tw, n_chunks = (L.nz + s->chunk_z - 1) / s->chunk_z;
-  const int nf = tiles * n_chunks;
-  std::vector<int> fl;
-  const int rc = rz_flags(s, tw, tiles, n_chunks, &fl);
-  if (rc != TETM_OK) return rc;
+  const int nf = (int)fl.size(), n_chunks = nf / tiles;
   cudaError_t e = cudaSuccess;
   std::vector<int> w, first((size_t)n_chunks + 1, 0);
   long long processed = 0;
@@ -2421,29 +2421,31 @@ int rz_rebuild_work(tetm_rz* s) try {
     processed += (long long)width * planes;
   }
   first[(size_t)n_chunks] = (int)w.size();
-  int* work = nullptr;
-  if (!w.empty()) {
-    e = cudaMalloc(&work, sizeof(int) * w.size());
-    if (e == cudaSuccess) e = cudaMemcpy(work, w.data(), sizeof(int) * w.size(), cudaMemcpyHostToDevice);
-  }
-  if (e == cudaSuccess && s->esz == 4 && tw == kTile2 && !s->changes) {  // once: they depend on the geometry only
+  const bool changes = s->esz == 4 && tw == kTile2 && !s->changes;  // once: they depend on the geometry only
+  if (changes) {
     s->change_words = (int)((L.rows + 31) / 32);
     const long long warps = (long long)tiles * s->change_words;
     e = cudaMalloc(&s->changes, sizeof(unsigned) * (size_t)warps);
     if (e == cudaSuccess) {
       rz_mask_changes<<<(unsigned)((warps + 7) / 8), 256, 0, s->st>>>(s->mask, L, tiles, s->change_words, s->changes);
       e = cudaGetLastError();
-      // (the caller may step on another stream next: tetm_rz_set_stream)
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-      if (e != cudaSuccess) {
-        cudaFree(s->changes);
-        s->changes = nullptr;
-      }
     }
   }
+  int* work = nullptr;
+  if (e == cudaSuccess && !w.empty()) {
+    e = cudaMalloc(&work, sizeof(int) * w.size());
+    if (e == cudaSuccess) e = cudaMemcpy(work, w.data(), sizeof(int) * w.size(), cudaMemcpyHostToDevice);
+  }
+  // (the caller may step on another stream next: tetm_rz_set_stream)
+  if (changes && e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   if (e != cudaSuccess) {
+    const int rc = rz_fail(e);
     cudaFree(work);
-    return rz_fail(e);
+    if (changes) {
+      cudaFree(s->changes);
+      s->changes = nullptr;
+    }
+    return rc;
   }
   cudaFree(s->work);
   s->work = work;
@@ -2455,6 +2457,13 @@ int rz_rebuild_work(tetm_rz* s) try {
   s->processed = processed * s->n_modes;
   s->work_dirty = false;
   return TETM_OK;
+}
+
+int rz_rebuild_work(tetm_rz* s) try {
+  const int tw = rz_tile_width(s), tiles = (s->L.nr + 1 + tw - 1) / tw;
+  std::vector<int> fl;
+  const int rc = rz_flags(s, tw, tiles, s->chunk_z, &fl);
+  return rc == TETM_OK ? rz_take_list(s, tw, tiles, fl) : rc;
 } catch (const std::bad_alloc&) {
   return TETM_E_NOMEM;
 }
@@ -2490,20 +2499,33 @@ int rz_reshape(tetm_rz* s, int kernel, int chunk_z, bool retile) {
 // single float32 steps (a call of one step), bulk-copy sweep on 56-entry windows
 // against the asynchronous-copy one with 32 planes, 93 x 771 28.6 | 6.3, 512 x
 // 4096 90 | 74.
+// The flags of two planes each give those of every even length: a thread scans
+// an item's mask bytes one by one, up to 1792 of an empty one of 32 planes.
 int rz_default_chunk(tetm_rz* s) try {
-  const int tw = rz_tile_width(s), nz = s->L.nz;
-  const int tiles = (s->L.nr + 1 + tw - 1) / tw, n_chunks = (nz + s->chunk_z - 1) / s->chunk_z;
-  const int least = s->esz == 8 ? 8 : s->mat ? 4 : 2;  // (the one-step sweeps start later)
-  // (one allocation for the flags of every chunk length there can be and the hulls of rz_build_band)
-  int rc = rz_reserve_flags(s, std::max(tiles * ((nz + least - 1) / least), 2 * nz));
+  const int tw = rz_tile_width(s), tiles = (s->L.nr + 1 + tw - 1) / tw, nz = s->L.nz;
+  std::vector<int> two;
+  // (one allocation for them and the hulls of rz_build_band)
+  int rc = rz_reserve_flags(s, std::max(tiles * ((nz + 1) / 2), 2 * nz));
+  if (rc == TETM_OK) rc = rz_flags(s, tw, tiles, 2, &two);
   if (rc != TETM_OK) return rc;
-  std::vector<int> fl;
-  rc = rz_flags(s, tw, tiles, n_chunks, &fl);
-  if (rc != TETM_OK) return rc;
-  const long long planes = (long long)std::count_if(fl.begin(), fl.end(), [](int f) { return f != 0; }) * s->n_modes * s->chunk_z;
-  const int cz = (int)std::min(16LL, std::max((long long)least, planes / (4LL * 4 * std::max(1, s->resident)) / 2 * 2));
-  if (cz < nz) s->chunk_z = cz;
-  return rz_rebuild_work(s);
+  auto flags_of = [&](int cz) {
+    std::vector<int> fl((size_t)tiles * ((nz + cz - 1) / cz), 0);
+    for (int r = 0, rows = (nz + 1) / 2; r < rows; ++r) {
+      int* to = fl.data() + (size_t)(r / (cz / 2)) * tiles;
+      const int* from = two.data() + (size_t)r * tiles;
+      for (int t = 0; t < tiles; ++t) to[t] |= from[t];
+    }
+    return fl;
+  };
+  std::vector<int> fl = flags_of(s->chunk_z);
+  const long long planes = (long long)std::count(fl.begin(), fl.end(), 1) * s->n_modes * s->chunk_z;
+  const long long least = s->esz == 8 ? 8 : s->mat ? 4 : 2;  // (the one-step sweeps start later)
+  const int cz = (int)std::min(16LL, std::max(least, planes / (4LL * 4 * std::max(1, s->resident)) / 2 * 2));
+  if (cz < nz) {
+    s->chunk_z = cz;
+    fl = flags_of(cz);
+  }
+  return rz_take_list(s, tw, tiles, fl);
 } catch (const std::bad_alloc&) {
   return TETM_E_NOMEM;
 }
