@@ -112,12 +112,13 @@ __device__ double face_minv(const GeomIn& g, int axis, long i, long j, long k) {
 
 // Per-entry arrays of a component (material runs; nullptr where not kept): the
 // steps' coefficient s M^-1 and, for the balances, which would otherwise divide
-// at every use, M^-1 and M in float64 (float64 fields) or M and a2 M^-1 as
-// (hi, lo) float32 pairs whose sum is the float64 value to 2^-48 (float32).
+// at every use, M^-1 in float64 (float64 fields; M by recip_coef) or M and a2
+// M^-1 as (hi, lo) float32 pairs whose sum is the float64 value to 2^-48
+// (float32).
 struct EntryOut {
   void* u;
   double s;
-  double *minv, *m;
+  double* minv;
   float2 *mp, *ap;
   double a2;
 };
@@ -134,7 +135,6 @@ __device__ __forceinline__ void put_entry(const EntryOut& o, long long id, doubl
   static_cast<T*>(o.u)[id] = (T)(o.s * v);
   if constexpr (sizeof(T) == 8) {
     o.minv[id] = v;
-    o.m[id] = 1.0 / v;
   } else {
     o.mp[id] = pair(1.0 / v);
     if (o.ap) o.ap[id] = pair(o.a2 * v);
@@ -185,6 +185,14 @@ __global__ void __launch_bounds__(256) build_geometry(GeomIn g, Layout L, int k_
   }
   const int n = __syncthreads_count(m != 0 && k >= 0 && k < g.nz);  // (the cell (i, j, k) is open: i < nx, j < ny)
   if (threadIdx.x == 0 && n) atomicAdd(active, (unsigned long long)n);
+}
+
+// M = 1/M^-1 per entry (0 where M^-1 is 0: an entry without a field), float64
+// fields: a pass of its own, so that the cell arrays are released before the M
+// arrays are made and a solve needs no more memory to be created than to be kept
+__global__ void recip_coef(const double* minv, long long n, double* out) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < n) out[q] = minv[q] != 0.0 ? 1.0 / minv[q] : 0.0;
 }
 
 // flags |= 1: a value is not a finite number >= 1, |= 2: not all are equal
@@ -1044,13 +1052,12 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
       zeroed(&s->ua[c], n * s->esz);
       if (s->esz == 8) {
         zeroed((void**)&s->minv_a[c], n * sizeof(double));
-        zeroed((void**)&s->m_a[c], n * sizeof(double));
       } else {
         zeroed((void**)&s->mp[c], n * sizeof(float2));
         if (a2) zeroed((void**)&s->ap[c], n * sizeof(float2));
       }
       eo.c[c] = EntryOut{s->ua[c],    (c == kEZ || c == kHZ) ? 2.0 * s->alpha : s->alpha,
-                         s->minv_a[c], s->m_a[c], s->mp[c], s->ap[c], s->alpha * s->alpha};
+                         s->minv_a[c], s->mp[c], s->ap[c], s->alpha * s->alpha};
     }
   }
   // upload the cell arrays, build the mask (and the per-entry arrays) on the device
@@ -1111,6 +1118,13 @@ int create_impl(const tetm_grid* g, int k_lo, int nz_all, const double* eps_r, c
   dev_free(cnt, s->stream);
   dev_free(dpec, s->stream);
   for (double* d : dcell) dev_free(d, s->stream);
+  if (!uniform && s->esz == 8)
+    for (int c = 0; c < 6 && rc == TETM_OK; ++c) {
+      rc = dalloc(s, (void**)&s->m_a[c], sizeof(double) * (size_t)s->L.count);
+      if (rc != TETM_OK) break;
+      recip_coef<<<(unsigned)((s->L.count + 255) / 256), 256, 0, s->stream>>>(s->minv_a[c], s->L.count, s->m_a[c]);
+      if (cudaGetLastError() != cudaSuccess) rc = TETM_E_CUDA;
+    }
   // per-component constants for the uniform case (vacuum or one material)
   const double dx = g->dx, dy = g->dy, dz = g->dz;
   s->minv_c[kEX] = dx / (kEps0 * eps_u * dy * dz);
